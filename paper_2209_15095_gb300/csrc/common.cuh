@@ -217,6 +217,43 @@ __device__ __forceinline__ void grid_totals(const double* part, double (&out)[NQ
   __syncthreads();
 }
 
+// Exact widening to FP64.  For a float, normal values are widened on the
+// integer pipe (rebias the exponent, shift the mantissa): the hardware
+// conversion is an FP64-pipe instruction, which costs as much as an FMA.
+// Zero, subnormal, infinite and NaN values take the hardware conversion.
+__device__ __forceinline__ double to_f64(double x) { return x; }
+__device__ __forceinline__ double to_f64(float x) {
+  const unsigned f = __float_as_uint(x);
+  const unsigned e = (f >> 23) & 0xffu;
+  if (e - 1u < 254u) {
+    const unsigned hi = (f & 0x80000000u) | ((e + 896u) << 20) | ((f & 0x7fffffu) >> 3);
+    const unsigned lo = (f & 7u) << 29;
+    return __hiloint2double((int)hi, (int)lo);
+  }
+  return (double)x;
+}
+
+// Rounding of an FP64 value to FP32, to nearest with ties to even (IEEE
+// 754), on the integer pipe where the result is a normal float: the FP32
+// exponent is the FP64 one rebiased (1023 -> 127), the 23 mantissa bits are
+// the top of the 52, and the 29 bits dropped decide the rounding (above
+// half: up; exactly half: up when the kept mantissa is odd).  A carry out
+// of the mantissa increments the exponent, and one out of the largest
+// exponent gives the infinity bit pattern, as the rounding rule does.
+// Results that would be subnormal, zero, infinite or NaN take the hardware
+// conversion (an FP64-pipe instruction, as costly as an FMA on this GPU).
+__device__ __forceinline__ float to_f32_rn(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned ex = (hi >> 20) & 0x7ffu;
+  if (ex - 897u < 254u) {
+    const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned r = lo & 0x1fffffffu;
+    const unsigned up = (r > 0x10000000u || (r == 0x10000000u && (m & 1u))) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (((ex - 896u) << 23) + m + up));
+  }
+  return (float)x;
+}
+
 // FP32 error-free accumulation of products (TwoProduct via fma + TwoSum,
 // Ogita, Rump & Oishi 2005): s + c carries the sum to about twice single
 // precision.  Intrinsics keep the compiler from contracting or reassociating.

@@ -30,6 +30,7 @@
 
 #include "common.cuh"
 #include "levelset.cuh"
+#include "weno_int.cuh"
 
 namespace etd {
 
@@ -75,6 +76,7 @@ struct LsArgs {
   int mode;
   int reinit;
   int mixed;  // FP32 WENO/Godunov arithmetic away from the interface
+  WenoInt wi;  // constants of the integer WENO5 form
 };
 
 LevelsetBufs levelset_carve(const GridDev& g, const std::function<char*(size_t)>& take) {
@@ -207,129 +209,157 @@ __device__ __forceinline__ C weno5_upwind(const Weno5Terms<C>& t, C r0, C r1, bo
   return max0(positive ? dm : -dm, positive ? -dp : dp);
 }
 
-// Constants of the Godunov evaluations of one grid, computed once.
-struct WenoK {
-  double epsw;     // eps' on undivided FP64 differences: 4 eps h^2
-  double inv_h;    // 1 / h
-  double inv_h12;  // 1 / (12 h): the scale of the FP64 result
+// One axis of the Godunov |grad phi|, scaled by 12, in FP64: the form for
+// values out of the integer form's range (weno_int.cuh), h 12 |.| from
+// undivided differences with eps' = 4 eps h^2.
+__device__ __noinline__ double godunov_mx_f64(const double* f, bool positive, double h) {
+  double q[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) q[k] = f[k + 1] - f[k];
+  const Weno5Terms<double> t = weno5_terms<double>(q, 4.0 * WENO_EPS * h * h);
+  return weno5_upwind<double>(t, 4.0 / t.W[0], 4.0 / t.W[1], positive);
+}
+
+// The values of phi, p_1 and p_2 (k = 0, 1, 2) as the stages' stencils read
+// them: FP64, 64-bit integers (weno_int.cuh) and FP32.  A value is converted
+// once, where it is written, instead of at each of the 6N + 1 nodes that
+// read it: a conversion between FP64 and FP32 or integers issues at the FP64
+// rate.  The copies live in the extension's buffers, which are free from the
+// Stefan speed on.
+__device__ __forceinline__ double* stage_f64(const LsArgs& a, int k) { return k == 0 ? a.phi : k == 1 ? a.b.p1 : a.b.p2; }
+__device__ __forceinline__ i64* stage_int(const LsArgs& a, int k) { return reinterpret_cast<i64*>(a.b.q[k]); }
+__device__ __forceinline__ float* stage_f32(const LsArgs& a, int k) {
+  return k == 2 ? reinterpret_cast<float*>(a.b.q[4]) : reinterpret_cast<float*>(a.b.q[3]) + k * a.g.size;
+}
+// Which copies a call's stages read: FP64 runs integers; mixed runs FP32, and
+// integers too while some entries keep FP64 accuracy (the reinitialisation).
+enum : int { COPY_INT = 1, COPY_F32 = 2 };
+__device__ __forceinline__ void stage_put(const LsArgs& a, int copies, int k, long long p, double v) {
+  stage_f64(a, k)[p] = v;
+  if (copies & COPY_INT) stage_int(a, k)[p] = to_fix(v, a.wi.eh);
+  if (copies & COPY_F32) stage_f32(a, k)[p] = to_f32_rn(v);
+}
+
+// A node of the update set as one lane evaluates it.
+template <int N>
+struct StageLane {
+  int p;         // grid index (-1: none)
+  int ax;        // split entries: the axis this lane evaluates
+  int ix[N];     // axis indices
+  bool inner;    // three nodes or more from every box face
+  double rate;   // advection: V; reinitialisation: S
+  double v[3];   // phi, p_1, p_2 at p
 };
 
-__device__ __forceinline__ WenoK weno_k(double h) {
-  WenoK k;
-  k.epsw = 4.0 * WENO_EPS * h * h;
-  k.inv_h = 1.0 / h;
-  k.inv_h12 = 1.0 / (12.0 * h);
-  return k;
-}
-
-// The seven values along axis d as six differences: FP64 undivided, or
-// FP32-mixed (values rounded to FP32, differences divided by h in FP32; an
-// eps' scaled by h^2 would leave the FP32 normal range).
-template <typename C, int N>
-__device__ __forceinline__ void axis_diffs(const GridDev& g, const double* __restrict__ src, long long p, const int* ix,
-                                           int d, double inv_h, C* q) {
-  double f[7];
-#pragma unroll
-  for (int k = -3; k <= 3; ++k) f[k + 3] = __ldcg(src + nbr(g, p, ix, d, k));
-  if constexpr (sizeof(C) == 8) {
-#pragma unroll
-    for (int k = -2; k <= 3; ++k) q[k + 2] = f[k + 3] - f[k + 2];
-  } else {
-    const C ih = C(inv_h);
-    C fc[7];
-#pragma unroll
-    for (int k = 0; k < 7; ++k) fc[k] = C(f[k]);
-#pragma unroll
-    for (int k = -2; k <= 3; ++k) q[k + 2] = (fc[k + 3] - fc[k + 2]) * ih;
-  }
-}
-
-// One axis of the Godunov |grad phi| (godunov, below), scaled by 12: the
-// upwind value from the WENO5 pair on the seven values along axis d.
-template <typename C, int N>
-__device__ __forceinline__ C godunov_mx(const GridDev& g, const double* __restrict__ src, long long p, const int* ix,
-                                        int d, bool positive, const WenoK& k) {
-  C q[6];
-  axis_diffs<C, N>(g, src, p, ix, d, k.inv_h, q);
-  const C epsw = sizeof(C) == 8 ? C(k.epsw) : C(4.0 * WENO_EPS);
-  const Weno5Terms<C> t = weno5_terms<C>(q, epsw);
-  if constexpr (sizeof(C) == 8) {
-    // W_s >= 10 eps'^4 (> 1e-70 for h > 1e-6) and for |q| < 1e18 the
-    // product stays finite: it neither underflows nor overflows in FP64
-    const C r = C(4) / (t.W[0] * t.W[1]);
-    return weno5_upwind<C>(t, t.W[1] * r, t.W[0] * r, positive);
-  } else {
-    return weno5_upwind<C>(t, C(4) / t.W[0], C(4) / t.W[1], positive);
-  }
-}
-
-// 4 / (W0 W1) of every axis.  When each product lies within 2^(+-1000/N)
-// one division serves all axes (prefix and suffix products of the others);
-// otherwise one division per axis.
+// offset of the node k steps along axis d
 template <int N>
-__device__ __forceinline__ void weno5_recips(const Weno5Terms<double>* t, double* r) {
-  constexpr unsigned LIM = 1000 / N;
-  double D[N];
-  bool shared = true;
+__device__ __forceinline__ long long step_of(const GridDev& g, const StageLane<N>& e, int d, int k) {
+  if (e.inner) return (long long)k * g.stride[d];
+  const int i = min(max(e.ix[d] + k, 0), g.n[d] - 1);
+  return (long long)(i - e.ix[d]) * g.stride[d];
+}
+
+// |grad phi| (Godunov, WENO5) at a node from the integer copy `src`; out of
+// range: in FP64 from `dsrc`.
+template <int N>
+__device__ __forceinline__ double grad_int(const LsArgs& a, const StageLane<N>& e, const i64* __restrict__ src,
+                                           const double* __restrict__ dsrc, bool positive) {
+  const GridDev& g = a.g;
+  i64 F[N][7];
+  const i64 own = __ldcg(src + e.p);
 #pragma unroll
   for (int d = 0; d < N; ++d) {
-    D[d] = t[d].W[0] * t[d].W[1];
-    const unsigned e = (unsigned)__double2hiint(D[d]) >> 20;  // biased exponent (D > 0)
-    shared = shared && e - (1023u - LIM) <= 2u * LIM;
+#pragma unroll
+    for (int k = -3; k <= 3; ++k) F[d][k + 3] = k == 0 ? own : __ldcg(src + e.p + step_of<N>(g, e, d, k));
   }
-  if (shared) {
-    double pre[N];
-    pre[0] = 1.0;
+  const int oh = (int)hi32((u64)own);
+  bool ok = (unsigned)(oh ^ (oh >> 31)) < FIX_OWN_HI;
+  U128 acc{0, 0};
 #pragma unroll
-    for (int d = 1; d < N; ++d) pre[d] = pre[d - 1] * D[d - 1];
-    const double rP = 4.0 / (pre[N - 1] * D[N - 1]);
-    double suf = 1.0;
-#pragma unroll
-    for (int d = N - 1; d >= 0; --d) {
-      r[d] = (rP * pre[d]) * suf;
-      suf *= D[d];
-    }
-  } else {
-#pragma unroll
-    for (int d = 0; d < N; ++d) r[d] = 4.0 / D[d];
+  for (int d = 0; d < N; ++d) {
+    i64 mx;
+    ok = weno_axis(F[d], positive, a.wi, mx) && ok;
+    acc = add128(acc, sq128(mx));
   }
+  if (ok) return grad_of(acc, a.wi);
+  double s = 0.0;
+  for (int d = 0; d < N; ++d) {
+    double f[7];
+    for (int k = -3; k <= 3; ++k) f[k + 3] = __ldcg(dsrc + e.p + step_of<N>(g, e, d, k));
+    const double mx = godunov_mx_f64(f, positive, g.h);
+    s = fma(mx, mx, s);
+  }
+  return sqrt(s) * (1.0 / (12.0 * g.h));
 }
 
-// Godunov |grad phi| at node p from array src; positive: outward motion.
-// FP64 (C = double): undivided differences, eps' scaled by h^2, every axis's
-// terms first so that one division serves the node, one factor 1/(12 h) at
-// the end.  FP32-mixed (C = float): WENO5 and Godunov in FP32, no FP64
-// arithmetic (this GPU issues one FP64 warp instruction per ~80 cycles per
-// SM sub-partition).
-template <typename C, int N>
-__device__ double godunov(const GridDev& g, const double* __restrict__ src, long long p, const int* ix,
-                          bool positive, const WenoK& k) {
-  if constexpr (sizeof(C) == 8) {
-    Weno5Terms<double> t[N];
+// The same with the node's axes on N consecutive lanes (all lanes of the warp
+// call this; lane d of the entry returns with the sum over its axes).
+template <int N>
+__device__ __forceinline__ double grad_int_split(const LsArgs& a, const StageLane<N>& e, const i64* __restrict__ src,
+                                                 const double* __restrict__ dsrc, bool positive) {
+  const GridDev& g = a.g;
+  U128 sq{0, 0};
+  bool ok = true;
+  if (e.p >= 0) {
+    i64 F[7], mx;
 #pragma unroll
-    for (int d = 0; d < N; ++d) {
-      double q[6];
-      axis_diffs<double, N>(g, src, p, ix, d, k.inv_h, q);
-      t[d] = weno5_terms<double>(q, k.epsw);
-    }
-    double r[N];
-    weno5_recips<N>(t, r);
-    double acc = 0.0;
-#pragma unroll
-    for (int d = 0; d < N; ++d) {
-      const double mx = weno5_upwind<double>(t[d], t[d].W[1] * r[d], t[d].W[0] * r[d], positive);
-      acc = fma(mx, mx, acc);
-    }
-    return sqrt(acc) * k.inv_h12;
-  } else {
-    float acc = 0.f;
-#pragma unroll
-    for (int d = 0; d < N; ++d) {
-      const float mx = godunov_mx<float, N>(g, src, p, ix, d, positive, k);
-      acc = fma(mx, mx, acc);
-    }
-    return (double)(sqrtf(acc) * (1.f / 12.f));
+    for (int k = -3; k <= 3; ++k) F[k + 3] = __ldcg(src + e.p + step_of<N>(g, e, e.ax, k));
+    const int oh = (int)hi32((u64)F[3]);
+    ok = weno_axis(F, positive, a.wi, mx) && (unsigned)(oh ^ (oh >> 31)) < FIX_OWN_HI;
+    sq = sq128(mx);
   }
+  const int base = (int)(threadIdx.x & 31) - e.ax;
+  U128 acc{0, 0};
+  bool all = true;
+#pragma unroll
+  for (int d = 0; d < N; ++d) {
+    const int l = (base + d) & 31;
+    acc = add128(acc, U128{__shfl_sync(0xffffffffu, sq.hi, l), __shfl_sync(0xffffffffu, sq.lo, l)});
+    all = __shfl_sync(0xffffffffu, (int)ok, l) && all;
+  }
+  double gr = grad_of(acc, a.wi);
+  if (__any_sync(0xffffffffu, !all)) {
+    double m = 0.0;
+    if (e.p >= 0) {
+      double f[7];
+      for (int k = -3; k <= 3; ++k) f[k + 3] = __ldcg(dsrc + e.p + step_of<N>(g, e, e.ax, k));
+      m = godunov_mx_f64(f, positive, g.h);
+    }
+    double s = 0.0;
+#pragma unroll
+    for (int d = 0; d < N; ++d) {
+      const double v = __shfl_sync(0xffffffffu, m, (base + d) & 31);
+      s = fma(v, v, s);
+    }
+    if (!all) gr = sqrt(s) * (1.0 / (12.0 * g.h));
+  }
+  return gr;
+}
+
+// The same in FP32 (mixed variant) from the FP32 copy: differences divided by
+// h (an eps' scaled by h^2 would leave the FP32 normal range).
+template <int N>
+__device__ __forceinline__ double grad_f32(const LsArgs& a, const StageLane<N>& e, const float* __restrict__ src,
+                                           bool positive, float inv_h) {
+  const GridDev& g = a.g;
+  float f[N][7];
+  const float own = __ldcg(src + e.p);
+#pragma unroll
+  for (int d = 0; d < N; ++d) {
+#pragma unroll
+    for (int k = -3; k <= 3; ++k) f[d][k + 3] = k == 0 ? own : __ldcg(src + e.p + step_of<N>(g, e, d, k));
+  }
+  float acc = 0.f;
+#pragma unroll
+  for (int d = 0; d < N; ++d) {
+    float q[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) q[k] = (f[d][k + 1] - f[d][k]) * inv_h;
+    const Weno5Terms<float> t = weno5_terms<float>(q, float(4.0 * WENO_EPS));
+    const float mx = weno5_upwind<float>(t, 4.f / t.W[0], 4.f / t.W[1], positive);
+    acc = fmaf(mx, mx, acc);
+  }
+  return to_f64(sqrtf(acc) * (1.f / 12.f));
 }
 
 // ------------------------------------------------------------ work lists
@@ -947,111 +977,142 @@ __device__ double stefan_speed_f32(const GridDev& g, const double* __restrict__ 
   return (double)((float)mu * fmaxf(0.f, (4.f * us[0] - us[1]) * (0.5f * inv_h)));
 }
 
-// TVD-RK3 on the nodes of T (list order); L(src, p) supplied by the caller.
-// Stage values p1/p2 hold phi off T (copied when the work set is built).
 // The stage list holds the work-list positions of the update set T: entries
-// pushed to the front first, then those pushed to the back (read in that
-// order), so that warps see one kind of entry (FP64 or FP32 arithmetic).
+// pushed to the front first (FP64 accuracy: the integer form), then those
+// pushed to the back (FP32; read in that order), so that warps see one kind.
 __device__ __forceinline__ void stage_push(const LsArgs& a, int i, bool front) {
   if (front) a.b.slist[atomicAdd(&a.b.count[1], 1)] = i;
   else a.b.slist[a.g.size - 1 - atomicAdd(&a.b.count[2], 1)] = i;
 }
 
-// How the front entries of the stage list (the FP64 ones) are dealt to warps:
-// a lane per entry, or an axis per lane.
-enum : int { SPLIT_NONE = 0, SPLIT_ALL = 1 };
-
-// One TVD-RK3 step over the stage list.  Front entries go a lane per entry
-// (SPLIT_NONE) or have their N axes evaluated on N lanes each (SPLIT_ALL,
-// 32 / N entries per warp): the per-axis terms come back by shuffles and are
-// summed in axis order as in godunov (which differs only in sharing one
-// division among the axes, i.e. in rounding), and a warp issues a third (3D)
-// of the FP64 instructions of a warp of whole entries.  This GPU issues about
-// one FP64 warp instruction per 80 cycles per SM sub-partition whatever the
-// warp's active lanes, so where few FP64 entries leave at most a warp or two
-// per sub-partition, split warps finish sooner.  Back entries (FP32 ones) go
-// a lane per entry.  L(src, p, ix, i, front) gives the update value of a
-// whole entry, LAx(src, p, ix, i, d) the axis term of a split one and
-// LFin(i, acc) its update value.
-template <int N, typename LFn, typename LAx, typename LFin>
-__device__ bool rk3(const LsArgs& a, LsCtx& c, double dt, bool clamp_last, int split, LFn L, LAx LAxis,
-                    LFin LFinal) {
-  const GridDev& g = a.g;
-  const int nf = __ldcg(a.b.count + 1), nb = __ldcg(a.b.count + 2);
-  const double G = BAND * g.h;
-  // 32-entry chunks dealt round-robin over the CTAs: every SM gets its share
-  // of each kind while a warp reads 32 consecutive entries.  Chunk order:
-  // whole front, split front, back.
-  const int lane = threadIdx.x & 31;
-  const long long warp0 = (long long)blockIdx.x + (long long)gridDim.x * (threadIdx.x >> 5);
-  const long long wstride = (long long)gridDim.x * (blockDim.x >> 5);
-  constexpr int NPW = 32 / N;  // split entries per warp
-  const long long nwf = split == SPLIT_NONE ? nf : 0;
-  const long long cw = (nwf + 31) / 32;
-  const long long cf = ((long long)nf - nwf + NPW - 1) / NPW;
-  const long long nchunk = cw + cf + ((long long)nb + 31) / 32;
-  for (int stage = 0; stage < 3; ++stage) {
-    const double* src = stage == 0 ? a.phi : (stage == 1 ? a.b.p1 : a.b.p2);
-    auto update = [&](long long p, double Lv) {
-      const double ph = a.phi[p];
-      if (stage == 0) {
-        a.b.p1[p] = ph + dt * Lv;
-      } else if (stage == 1) {
-        a.b.p2[p] = 0.75 * ph + 0.25 * (__ldcg(a.b.p1 + p) + dt * Lv);
-      } else {
-        double v = fma(1.0 / 3.0, ph, 2.0 / 3.0 * (__ldcg(a.b.p2 + p) + dt * Lv));
-        if (clamp_last) v = fmin(fmax(v, -G), G);
-        a.phi[p] = v;
-      }
-    };
-    for (long long chunk = warp0; chunk < nchunk; chunk += wstride) {
-      if (chunk >= cw && chunk < cw + cf) {
-        const int sub = lane / N, d = lane - sub * N;
-        const long long j = nwf + (chunk - cw) * NPW + sub;
-        const bool valid = sub < NPW && j < nf;
-        long long i = 0, p = 0;
-        double mx = 0.0;
-        if (valid) {
-          i = __ldcg(a.b.slist + j);
-          p = __ldcg(a.b.list + i);
-          int ix[N];
-          unpack<N>(a.b.lcoord[i], ix);
-          mx = LAxis(src, p, ix, i, d);
-        }
-        double acc = 0.0;
+// How the stage list is dealt: chunks of warps' work, round-robin over the
+// CTAs (every SM gets its share of each kind).  Front entries go a lane each,
+// or, where all of them then still make one round of the warps at most, an
+// axis per lane (32 / N entries per warp): the same instructions in all, a
+// third (3D) of the dependent chain per warp.  Back entries go a lane each.
+template <int N>
+struct StageDeal {
+  static constexpr int NPW = 32 / N;  // split entries per warp
+  int nf, nb, cf, nchunk, warp0, wstride;
+  bool split;
+  __device__ __forceinline__ StageDeal(const LsArgs& a) {
+    nf = __ldcg(a.b.count + 1);
+    nb = __ldcg(a.b.count + 2);
+    warp0 = (int)blockIdx.x + (int)gridDim.x * (int)(threadIdx.x >> 5);
+    wstride = (int)gridDim.x * (int)(blockDim.x >> 5);
+    const int cb = (nb + 31) / 32, cs = (nf + NPW - 1) / NPW;
+    split = cs + cb <= wstride;
+    cf = split ? cs : (nf + 31) / 32;
+    nchunk = cf + cb;
+  }
+  // this lane's entry of a chunk
+  __device__ __forceinline__ StageLane<N> lane(const LsArgs& a, int chunk, const double* rates) const {
+    const int l = threadIdx.x & 31;
+    StageLane<N> e;
+    e.p = -1;
+    e.ax = 0;
+    e.rate = 0.0;
+    long long j;
+    bool has;
+    if (chunk < cf && split) {
+      const int sub = l / N;
+      e.ax = l - sub * N;
+      j = (long long)chunk * NPW + sub;
+      has = sub < NPW && j < nf;
+    } else {
+      j = 32ll * (chunk < cf ? chunk : chunk - cf) + l;
+      has = j < (chunk < cf ? nf : nb);
+    }
+    if (has) {
+      const int i = __ldcg(a.b.slist + (chunk < cf ? j : a.g.size - 1 - j));
+      e.p = __ldcg(a.b.list + i);
+      unpack<N>(__ldcg(a.b.lcoord + i), e.ix);
+      e.rate = __ldcg(rates + i);
+      e.inner = true;
 #pragma unroll
-        for (int e = 0; e < N; ++e) {
-          const double v = __shfl_sync(0xffffffffu, mx, sub * N + e);
-          acc = fma(v, v, acc);
-        }
-        if (valid && d == 0) update(p, LFinal(i, acc));
-        continue;
+      for (int d = 0; d < N; ++d) e.inner = e.inner && e.ix[d] >= 3 && e.ix[d] < a.g.n[d] - 3;
+    }
+    return e;
+  }
+};
+
+// One TVD-RK3 step on the stage list, phi_t = rate(|grad phi|).  REINIT:
+// phi_t = S (1 - |grad phi|), upwinded by the sign of S; else phi_t =
+// -V |grad phi|.  A warp's first chunk keeps its entries (position, rate, own
+// values) in `e0` over the steps of a call, so that a stage starts with its
+// stencil loads; larger lists load the entries of the further chunks.
+template <int N, bool REINIT>
+__device__ bool rk3(const LsArgs& a, LsCtx& c, const StageDeal<N>& deal, StageLane<N>& e0, const double* rates,
+                    int copies, double dt, bool clamp_last) {
+  const double G = BAND * a.g.h;
+  const float inv_h = (float)(1.0 / a.g.h);
+  for (int stage = 0; stage < 3; ++stage) {
+    const auto run = [&](StageLane<N>& e, int chunk) {
+      const bool positive = !REINIT || e.rate > 0.0;
+      double gr = 0.0;
+      if (chunk >= deal.cf) {
+        if (e.p >= 0) gr = grad_f32<N>(a, e, stage_f32(a, stage), positive, inv_h);
+      } else if (deal.split) {
+        gr = grad_int_split<N>(a, e, stage_int(a, stage), stage_f64(a, stage), positive);
+      } else if (e.p >= 0) {
+        gr = grad_int<N>(a, e, stage_int(a, stage), stage_f64(a, stage), positive);
       }
-      const bool front = chunk < cw;
-      const long long j = front ? 32 * chunk + lane : 32 * (chunk - cw - cf) + lane;
-      if (j >= (front ? nwf : (long long)nb)) continue;
-      const long long i = __ldcg(a.b.slist + (front ? j : g.size - 1 - j));
-      const long long p = __ldcg(a.b.list + i);
-      int ix[N];
-      unpack<N>(a.b.lcoord[i], ix);
-      update(p, L(src, p, ix, i, front));
+      if (e.p < 0 || e.ax != 0) return;
+      const double L = REINIT ? fma(-e.rate, gr, e.rate) : -e.rate * gr;
+      if (stage == 0) {
+        e.v[1] = e.v[0] + dt * L;
+      } else if (stage == 1) {
+        e.v[2] = 0.75 * e.v[0] + 0.25 * (e.v[1] + dt * L);
+      } else {
+        double v = fma(1.0 / 3.0, e.v[0], 2.0 / 3.0 * (e.v[2] + dt * L));
+        if (clamp_last) v = fmin(fmax(v, -G), G);
+        e.v[0] = v;
+      }
+      const int to = stage == 2 ? 0 : stage + 1;
+      stage_put(a, copies, to, e.p, e.v[to]);
+    };
+    if (deal.warp0 < deal.nchunk) run(e0, deal.warp0);
+    for (int chunk = deal.warp0 + deal.wstride; chunk < deal.nchunk; chunk += deal.wstride) {
+      StageLane<N> e = deal.lane(a, chunk, rates);
+      if (e.p >= 0) {
+        e.v[0] = a.phi[e.p];
+        if (stage == 1) e.v[1] = a.b.p1[e.p];
+        if (stage == 2) e.v[2] = a.b.p2[e.p];
+      }
+      run(e, chunk);
     }
     if (!grid_barrier(a.st, c.bar, 30 + stage)) return false;
   }
   return true;
 }
 
-// copy phi into the RK stage buffers on the work list
-template <int N>
-__device__ void stage_init(const LsArgs& a) {
-  const int n = __ldcg(a.b.count);
-  const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x, gth = (long long)gridDim.x * blockDim.x;
-  for (long long i = gtid; i < n; i += gth) {
-    const long long p = __ldcg(a.b.list + i);
-    const double v = a.phi[p];
-    a.b.p1[p] = v;
-    a.b.p2[p] = v;
+// phi into the stages' copies at a work-list node
+__device__ __forceinline__ void stage_init(const LsArgs& a, int copies, long long p) {
+  const double v = a.phi[p];
+  a.b.p1[p] = v;
+  a.b.p2[p] = v;
+  if (copies & COPY_INT) {
+    const i64 f = to_fix(v, a.wi.eh);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) stage_int(a, k)[p] = f;
   }
+  if (copies & COPY_F32) {
+    const float f = to_f32_rn(v);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) stage_f32(a, k)[p] = f;
+  }
+}
+
+// K steps of rk3 on the stage list
+template <int N, bool REINIT>
+__device__ bool rk3_steps(const LsArgs& a, LsCtx& c, const double* rates, int copies, int K, double dt) {
+  const StageDeal<N> deal(a);
+  StageLane<N> e0 = deal.lane(a, deal.warp0, rates);
+  e0.v[0] = e0.p >= 0 ? a.phi[e0.p] : 0.0;
+  e0.v[1] = e0.v[2] = 0.0;
+  for (int it = 0; it < K; ++it)
+    if (!rk3<N, REINIT>(a, c, deal, e0, rates, copies, dt, it == K - 1)) return false;
+  return true;
 }
 
 template <int N>
@@ -1065,42 +1126,21 @@ __device__ bool reinitialise(const LsArgs& a, LsCtx& c) {
   const int n = __ldcg(a.b.count);
   const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x, gth = (long long)gridDim.x * blockDim.x;
   const double h = g.h;
-  // mixed path: FP64 within h of the interface (|phi_0| < h, i.e.
-  // |S| < 1/sqrt(2)), FP32 WENO/Godunov arithmetic further out; the two
-  // kinds go to the two ends of the stage list, the FP64 ones an axis per
-  // lane (see rk3)
+  // mixed path: FP64 accuracy within h of the interface (|phi_0| < h, i.e.
+  // |S| < 1/sqrt(2)), FP32 WENO/Godunov arithmetic further out
   const double near_s = 1.0 / sqrt(2.0);
+  const int copies = a.mixed ? COPY_INT | COPY_F32 : COPY_INT;
   for (long long i = gtid; i < n; i += gth) {
     const long long p = __ldcg(a.b.list + i);
     const double ph = a.phi[p];
     const double S = ph / sqrt(ph * ph + h * h);
     a.b.S0[i] = S;
     if (a.b.lflag[i] & F_T) stage_push(a, (int)i, !a.mixed || fabs(S) < near_s);
+    stage_init(a, copies, p);
   }
-  stage_init<N>(a);
   if (!grid_barrier(a.st, c.bar, 40)) return false;
   const int K = (int)ceil(12.0 * sqrt((double)N));
-  const double dtau = 0.5 * h / sqrt((double)N);
-  const WenoK wk = weno_k(h);
-  auto L = [&](const double* src, long long p, const int* ix, long long i, bool fp64) {
-    const double S = __ldcg(a.b.S0 + i);
-    const double gr =
-        fp64 ? godunov<double, N>(g, src, p, ix, S > 0.0, wk) : godunov<float, N>(g, src, p, ix, S > 0.0, wk);
-    return fma(-S, gr, S);  // -S (|grad phi| - 1)
-  };
-  // FP64 entries an axis per lane (see rk3)
-  auto LAx = [&](const double* src, long long p, const int* ix, long long i, int d) {
-    return godunov_mx<double, N>(g, src, p, ix, d, __ldcg(a.b.S0 + i) > 0.0, wk);
-  };
-  auto LFin = [&](long long i, double acc) {
-    const double S = __ldcg(a.b.S0 + i);
-    return fma(-S, sqrt(acc) * wk.inv_h12, S);
-  };
-  const int split = a.mixed ? SPLIT_ALL : SPLIT_NONE;
-  for (int it = 0; it < K; ++it) {
-    if (!rk3<N>(a, c, dtau, it == K - 1, split, L, LAx, LFin)) return false;
-  }
-  return true;
+  return rk3_steps<N, true>(a, c, a.b.S0, copies, K, 0.5 * h / sqrt((double)N));
 }
 
 template <int N>
@@ -1208,8 +1248,6 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
     a.b.gidx[p] = (int)i;
     U[0][p] = (f & F_V0) ? a.u[p] : 0.0;
     UN[0][p] = un;
-    a.b.p1[p] = a.phi[p];
-    a.b.p2[p] = a.phi[p];
   }
   {
     const int lane = threadIdx.x & 31;
@@ -1304,6 +1342,7 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
     double vm = 0.0;
     for (long long i = gtid; i < n; i += gth) {
       const long long p = __ldcg(a.b.list + i);
+      stage_init(a, a.mixed ? COPY_F32 : COPY_INT, p);
       if (!(a.b.lflag[i] & F_T)) continue;
       int ix[N];
       unpack<N>(a.b.lcoord[i], ix);
@@ -1356,7 +1395,7 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
         V = a.mu * fmax(0.0, (4.0 * us[0] - us[1]) * inv_2h);
       }
       a.b.V[i] = V;
-      stage_push(a, (int)i, true);
+      stage_push(a, (int)i, !a.mixed);
       vm = fmax(vm, V);
     }
     for (int o = 16; o > 0; o >>= 1) vm = fmax(vm, __shfl_xor_sync(0xffffffffu, vm, o));
@@ -1377,17 +1416,7 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
       *a.b.nsub = nsub;
       a.b.info[2] = nsub;
     }
-    const double dts = a.dt / nsub;
-    const WenoK wk = weno_k(h);
-    auto L = [&](const double* s, long long p, const int* ix, long long i, bool) {
-      const double gr = a.mixed ? godunov<float, N>(g, s, p, ix, true, wk) : godunov<double, N>(g, s, p, ix, true, wk);
-      return -__ldcg(a.b.V + i) * gr;
-    };
-    for (int sub = 0; sub < nsub; ++sub) {
-      auto LAx = [&](const double*, long long, const int*, long long, int) { return 0.0; };
-      auto LFin = [&](long long, double) { return 0.0; };
-      if (!rk3<N>(a, c, dts, sub == nsub - 1, SPLIT_NONE, L, LAx, LFin)) return;
-    }
+    if (!rk3_steps<N, false>(a, c, a.b.V, a.mixed ? COPY_F32 : COPY_INT, nsub, a.dt / nsub)) return;
   }
   if (a.reinit) reinitialise<N>(a, c);
 }
@@ -1422,6 +1451,7 @@ cudaError_t launch_levelset_advance(const GridDev& g, const LevelsetBufs& b, Dev
                                     cudaStream_t stream) {
   LsArgs a;
   a.mixed = mixed ? 1 : 0;
+  a.wi = weno_int(g.h, WENO_EPS);
   a.g = g;
   a.b = b;
   a.st = st;
@@ -1439,6 +1469,7 @@ cudaError_t launch_levelset_prepare(const GridDev& g, const LevelsetBufs& b, Dev
                                     bool mixed, cudaStream_t stream) {
   LsArgs a;
   a.mixed = mixed ? 1 : 0;
+  a.wi = weno_int(g.h, WENO_EPS);
   a.g = g;
   a.b = b;
   a.st = st;

@@ -1,0 +1,353 @@
+// HJ-WENO5 upwind differences in 64-bit integer arithmetic.
+//
+// This GPU issues an FP64 warp instruction once per 16 to 19 cycles per SM
+// (measured: DFMA 16.0, DADD 19.1), a 32 x 32 + 64 bit multiply-add once per
+// 0.55 and a 64-bit add once per 0.5.  The level-set stages are bound by FP64
+// issue, and the WENO5 weights are what they issue, so these run on the
+// integer pipe, at more than FP64 precision:
+//   * phi enters as F = phi 2^S with S = 54 - floor(log2 h) (h 2^S lies in
+//     [2^54, 2^55)), rounded once: exact for |phi| >= h / 4, off by at most
+//     half a unit 2^-S <= 2^-54 h below.  Differences are then exact, where
+//     FP64 rounds them to 2^-53 of their size (about h).
+//   * the squared smoothness terms s_k are exact 128-bit integers, their
+//     squares, pairwise products and the quotient 64-bit mantissas: the
+//     weights carry an error below 2^-53, against about 20 roundings of
+//     2^-53 in the FP64 form, and the result one of a few units.
+// The arithmetic covers |phi| < 16 2^floor(log2 h) (at least 8h; the tube's
+// phi is at most 6h + one node) with adjacent differences below 2^57 units
+// (at least 4h); other nodes take the FP64 form (weno_in_range).
+#pragma once
+#include <stdint.h>
+#include <string.h>
+
+#ifdef __CUDACC__
+#define ETD_HD __host__ __device__ __forceinline__
+#else
+#define ETD_HD inline
+#endif
+
+namespace etd {
+
+typedef unsigned long long u64;
+typedef long long i64;
+
+struct WenoInt {
+  int eh;            // floor(log2 h)
+  u64 e4hi, e4lo;    // (3/4) eps' 2^2S = 3e-6 (h 2^S)^2, 128 bits
+  double scale;      // 2^-S / (12 h): the gradient from 12 times itself in units
+  float epsf;        // (3/4) eps' in units of 2^eh, squared
+};
+
+constexpr i64 FIX_OUT = 1ll << 62;  // stored for a value out of range (either sign)
+constexpr unsigned FIX_OWN_HI = 1u << 26;   // |F| < 2^58
+constexpr unsigned FIX_DIFF_HI = 1u << 25;  // |difference| < 2^57
+
+inline WenoInt weno_int(double h, double eps) {
+  WenoInt w;
+  u64 b;
+  memcpy(&b, &h, 8);
+  w.eh = (int)((b >> 52) & 0x7ff) - 1023;
+  if (w.eh < -900 || w.eh > 900) {  // near the ends of the exponent range: nothing is in range
+    w.eh = -4000;
+    w.e4hi = w.e4lo = 0;
+    w.scale = 0.0;
+    w.epsf = 0.f;
+    return w;
+  }
+  const u64 one = (b & 0xfffffffffffffull) | (1023ull << 52);
+  double m;
+  memcpy(&m, &one, 8);  // h = m 2^eh, 1 <= m < 2
+  const double e4 = 3.0 * eps * m * m * 18014398509481984.0;  // times 2^54; the other 2^54 below
+  w.epsf = (float)(3.0 * eps * m * m);
+  const u64 i = (u64)e4;
+  w.e4hi = i >> 10;  // e4 2^54 = i 2^54: bits 54 and up
+  w.e4lo = i << 54;
+  // the fraction of e4 (i holds about 36 bits of its 53)
+  w.e4lo += (u64)((e4 - (double)i) * 18014398509481984.0);
+  const u64 sb = (u64)(1023 + w.eh - 54) << 52;
+  double s;
+  memcpy(&s, &sb, 8);  // 2^-S
+  w.scale = s / (12.0 * h);
+  return w;
+}
+
+// phi 2^S as a 64-bit integer, to nearest; FIX_OUT with phi's sign when
+// |phi| >= 16 2^eh, infinite or NaN.
+ETD_HD i64 to_fix(double f, int eh) {
+#ifdef __CUDA_ARCH__
+  const u64 b = (u64)__double_as_longlong(f);
+#else
+  u64 b;
+  memcpy(&b, &f, 8);
+#endif
+  const int k = (int)((b >> 52) & 0x7ff) - 1023 - eh;
+  const i64 sg = (i64)b >> 63;
+  if (k > 3) return (FIX_OUT ^ sg) - sg;
+  const int r = 4 - k;  // the mantissa times 2^6, shifted right by r >= 1
+  if (r > 60) return 0;
+  const u64 m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 6;
+  const i64 v = (i64)((m + (1ull << (r - 1))) >> r);
+  return (v ^ sg) - sg;
+}
+
+ETD_HD u64 wide(unsigned a, unsigned b, u64 c = 0) { return (u64)a * b + c; }
+ETD_HD unsigned hi32(u64 x) { return (unsigned)(x >> 32); }
+ETD_HD unsigned lo32(u64 x) { return (unsigned)x; }
+ETD_HD int clz32(unsigned x) {
+#ifdef __CUDA_ARCH__
+  return __clz((int)x);
+#else
+  return x ? __builtin_clz(x) : 32;
+#endif
+}
+// (h, l) <<< n, the upper word, 0 <= n < 32
+ETD_HD unsigned shfl32(unsigned l, unsigned h, int n) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_l(l, h, n);
+#else
+  return n ? (h << n) | (l >> (32 - n)) : h;
+#endif
+}
+
+struct U128 {
+  u64 hi, lo;
+};
+ETD_HD U128 add128(U128 a, U128 b) {
+  U128 r;
+#ifdef __CUDA_ARCH__
+  asm("add.cc.u64 %0, %2, %4;\n\taddc.u64 %1, %3, %5;"
+      : "=l"(r.lo), "=l"(r.hi)
+      : "l"(a.lo), "l"(a.hi), "l"(b.lo), "l"(b.hi));
+#else
+  r.lo = a.lo + b.lo;
+  r.hi = a.hi + b.hi + (r.lo < a.lo);
+#endif
+  return r;
+}
+// t^2, exact
+ETD_HD U128 sq128(i64 t) {
+  const i64 s = t >> 63;
+  const u64 a = (u64)((t ^ s) - s);
+  const unsigned h = hi32(a), l = lo32(a);
+  const u64 m = wide(h, l);
+  return add128(U128{wide(h, h), wide(l, l)}, U128{m >> 31, m << 33});
+}
+// x y of signed operands, exact (two's complement)
+ETD_HD U128 mul128(i64 x, i64 y) {
+  const unsigned xh = hi32((u64)x), xl = lo32((u64)x), yh = hi32((u64)y), yl = lo32((u64)y);
+  const u64 ll = wide(xl, yl);
+  const u64 m1 = wide(xl, yh, ll >> 32);
+  const u64 m2 = wide(xh, yl, (u64)lo32(m1));
+  u64 hi = wide(xh, yh, m1 >> 32) + (m2 >> 32);
+  hi -= (u64)((x >> 63) & y) + (u64)((y >> 63) & x);
+  return U128{hi, (m2 << 32) | lo32(ll)};
+}
+// the upper 64 bits of x y, low by at most 2
+ETD_HD u64 mulhi_u(u64 x, u64 y) {
+  const u64 m1 = wide(hi32(x), lo32(y)), m2 = wide(lo32(x), hi32(y));
+  return wide(hi32(x), hi32(y), m1 >> 32) + (m2 >> 32);
+}
+ETD_HD u64 sqhi_u(u64 x) {
+  const u64 m = wide(hi32(x), lo32(x));
+  return wide(hi32(x), hi32(x), m >> 31);
+}
+ETD_HD u64 shr_sat(u64 x, int n) { return n > 63 ? 0ull : x >> n; }
+
+// leading 64 bits of s >= 2^64 (most significant bit set) and its leading zeros
+ETD_HD u64 normalise(U128 s, int& z) {
+  const unsigned w3 = hi32(s.hi), w2 = lo32(s.hi), w1 = hi32(s.lo), w0 = lo32(s.lo);
+  const bool top = w3 != 0;
+  const unsigned a = top ? w3 : w2, b = top ? w2 : w1, c = top ? w1 : w0;
+  const int n = clz32(a);
+  z = top ? n : n + 32;
+  return (u64)shfl32(b, a, n) << 32 | shfl32(c, b, n);
+}
+
+// 2^126 / w for w in [2^62, 2^63), to about 2^-58: a single-precision
+// reciprocal r0 of the leading bits, then r0 (1 + e + e^2) with
+// e = 1 - w r0 (|e| < 2^-21).
+ETD_HD u64 recip_u(u64 w) {
+  const unsigned wh = hi32(w);
+  float f;
+  unsigned fb = 0x3f000000u | ((wh - 0x40000000u) >> 7);  // w 2^-63, truncated
+#ifdef __CUDA_ARCH__
+  f = __uint_as_float(fb);
+  float rf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
+  rf = fminf(rf, 1.9999998f);
+  const unsigned r0 = (__float_as_uint(rf) & 0x7fffffu) << 8 | 0x80000000u;  // (1, 2) 2^31
+#else
+  memcpy(&f, &fb, 4);
+  float rf = 1.0f / f;
+  if (rf > 1.9999998f) rf = 1.9999998f;
+  unsigned rb;
+  memcpy(&rb, &rf, 4);
+  const unsigned r0 = (rb & 0x7fffffu) << 8 | 0x80000000u;
+#endif
+  // w r0 2^-32, about 2^62: p = w r0 >> 32 as 64 bits
+  const u64 p = wide(hi32(w), r0, wide(lo32(w), r0) >> 32);
+  const i64 e = (i64)((1ull << 62) - p);  // e 2^62, |e| < 2^42
+  const int eh = (int)(e >> 16);          // e 2^46, below 2^26
+  const i64 e1 = e + (((i64)eh * eh) >> 30);  // (e + e^2) 2^62
+  // r0 2^32 (1 + e1 2^-62), with |e1| < 2^42: r0 e1 2^-30 in two parts
+  const i64 c = ((i64)r0 * (int)(e1 >> 16) + (i64)(wide(r0, (unsigned)e1 & 0xffffu) >> 16)) >> 14;
+  return ((u64)r0 << 32) + (u64)c;
+}
+
+// (x y) >> 62 for |x| < 2^60 (signed) and a signed |y| < 2^63, to within 2 units
+ETD_HD i64 mul62(i64 x, i64 y) {
+  const U128 p = mul128(x, y);
+  return (i64)(p.hi << 2 | p.lo >> 62);
+}
+
+// 12 Phi(a, b, c, d) of Jiang & Peng's form (levelset.cu, weno5_terms) from
+// second differences in units 2^-S:
+//   12 Phi = (4 A X + V Y) / W,  A = d1 d2, B = d0 d2, C = d0 d1,
+//   W = A + 6 B + 3 C, V = 3 C - A - 6 B, X = a - 2b + c, Y = b - 2c + d,
+//   d_k = s_k^2,  s_0 = 4 (a-b)^2 + 3 b (2b-a), s_1 = 4 (b-c)^2 + 3 b c,
+//   s_2 = 4 (c-d)^2 + 3 c (2c-d), each plus 3/4 eps':
+// 3/4 of eps' + (13/3) t^2 + m^2, with 13 t^2 + 3 m^2 = 16 t^2 + 3 (m-t)(m+t).
+ETD_HD i64 weno_phi12(i64 a, i64 b, i64 c, i64 d, const WenoInt& k) {
+  const U128 e4{k.e4hi, k.e4lo};
+  const i64 t0 = a - b, t1 = b - c, t2 = c - d;
+  int z0, z1, z2;
+  const u64 s0 = normalise(add128(add128(sq128(2 * t0), mul128(3 * b, 2 * b - a)), e4), z0);
+  const u64 s1 = normalise(add128(add128(sq128(2 * t1), mul128(3 * b, c)), e4), z1);
+  const u64 s2 = normalise(add128(add128(sq128(2 * t2), mul128(3 * c, 2 * c - d)), e4), z2);
+  // squares, normalised; y_k: the larger, the smaller s_k
+  u64 d0 = sqhi_u(s0), d1 = sqhi_u(s1), d2 = sqhi_u(s2);
+  const int b0 = (i64)d0 >= 0, b1 = (i64)d1 >= 0, b2 = (i64)d2 >= 0;
+  d0 <<= b0;
+  d1 <<= b1;
+  d2 <<= b2;
+  const int y0 = 2 * z0 + b0, y1 = 2 * z1 + b1, y2 = 2 * z2 + b2;
+  const int y01 = y0 > y1 ? y0 : y1;
+  const int ym = (y01 > y2 ? y01 : y2) + 5;
+  u64 A = shr_sat(mulhi_u(d1, d2), ym - y0);
+  const u64 B = shr_sat(mulhi_u(d0, d2), ym - y1), C = shr_sat(mulhi_u(d0, d1), ym - y2);
+  const u64 AB = A + 6 * B, C3 = 3 * C;
+  u64 W = AB + C3;       // in [2^57, 2^62.4)
+  i64 V = (i64)(C3 - AB);
+  const int n = clz32(hi32(W)) - 1;
+  W <<= n;
+  A <<= n;
+  V = (i64)((u64)V << n);
+  // (4 A X + V Y) 2^-62, then the quotient
+  const i64 X = t0 - t1, Y = t1 - t2;
+  const U128 p = add128(mul128((i64)A, 4 * X), mul128(V, Y));
+  const i64 N = (i64)(p.hi << 2 | p.lo >> 62);
+  const i64 sg = N >> 63;
+  const u64 q = mulhi_u((u64)((N ^ sg) - sg), recip_u(W));  // |N| 2^126 / W 2^-64
+  return ((i64)q ^ sg) - sg;
+}
+
+// max(d, 0)-style upwind value of one axis, 12 max(d-, -d+, 0) for outward
+// motion (positive) or its mirror image, from the seven values F (units
+// 2^-S); false if a difference is out of range.  Only one side's weights are
+// evaluated: the larger of the two candidates a, b is decided on a
+// single-precision estimate of a - b = +-(d- + d+), whose error stays below
+// `tol` (the second differences enter truncated to 2^-22 2^eh, which moves a
+// weight by up to 0.3%: 5.1 2^-22 / sqrt(3e-6) per s_k, four-fold in the
+// quotient, rounded up to 2^-7 of the terms it multiplies); where that does
+// not decide, both sides are evaluated.  Equal values (all second
+// differences 0) need no decision.
+#ifdef __CUDACC__
+__device__ __forceinline__ bool weno_axis(const i64 (&F)[7], bool positive, const WenoInt& k, i64& out) {
+  const float epsf = k.epsf;
+  i64 q[6], e[5];
+  unsigned big = 0;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    q[i] = F[i + 1] - F[i];
+    const int h = (int)hi32((u64)q[i]);
+    big |= (unsigned)(h ^ (h >> 31));
+  }
+#pragma unroll
+  for (int i = 0; i < 5; ++i) e[i] = q[i + 1] - q[i];
+  const i64 cen = 7 * (q[2] + q[3]) - (q[1] + q[4]);
+  // the estimate, in units of 2^eh (f = 2^-22 leading words)
+  const float f0 = (float)(int)hi32((u64)e[0]) * 0x1p-22f, f1 = (float)(int)hi32((u64)e[1]) * 0x1p-22f,
+              f2 = (float)(int)hi32((u64)e[2]) * 0x1p-22f, f3 = (float)(int)hi32((u64)e[3]) * 0x1p-22f,
+              f4 = (float)(int)hi32((u64)e[4]) * 0x1p-22f;
+  const float ta = f0 - f1, tb = f1 - f2, tc = f2 - f3, td = f4 - f3;
+  const float Y = tb - tc, X0 = ta - tb, X1 = td + tc;
+  // s_k as in weno_phi12, eps' scaled to match
+  const float sb = fmaf(4.f * tb, tb, epsf), sc = fmaf(4.f * tc, tc, epsf);
+  const float bc = 3.f * f1, cd = 3.f * f3;
+  const float m0 = fmaf(4.f * ta, ta, fmaf(bc, 2.f * f1 - f0, epsf)), m1 = fmaf(bc, f2, sb),
+              m2 = fmaf(3.f * f2, 2.f * f2 - f3, sc);
+  const float p0 = fmaf(4.f * td, td, fmaf(cd, 2.f * f3 - f4, epsf)), p1 = fmaf(cd, f2, sc),
+              p2 = fmaf(3.f * f2, 2.f * f2 - f1, sb);
+  const auto phi = [](float s0, float s1, float s2, float X, float Yv) {
+    const float d0 = s0 * s0, d1 = s1 * s1, d2 = s2 * s2;
+    const float A = d1 * d2, AB = fmaf(6.f, d0 * d2, A), C3 = 3.f * (d0 * d1);
+    return __fdividef(fmaf(4.f * A, X, (C3 - AB) * Yv), AB + C3);
+  };
+  const float D = 2.f * ((float)(int)hi32((u64)cen) * 0x1p-22f) - phi(m0, m1, m2, X0, Y) + phi(p0, p1, p2, X1, Y);
+  const float tol = fmaf(0x1p-7f, 4.f * (fabsf(X0) + fabsf(X1)) + 2.f * fabsf(Y), 0x1p-14f);
+  const bool flat = (e[0] | e[1] | e[2] | e[3] | e[4]) == 0;  // d- = d+ = cen / 12
+  bool minus = (flat ? cen > 0 : D > 0.f) == positive;
+  bool both = !flat && !(fabsf(D) > tol);
+  i64 best = 0;
+  for (;;) {
+    const i64 ph = weno_phi12(minus ? e[0] : e[4], minus ? e[1] : e[3], e[2], minus ? e[3] : e[1], k);
+    const i64 v = minus ? cen - ph : -cen - ph;  // 12 d- or -12 d+
+    const i64 w = positive ? v : -v;
+    best = w > best ? w : best;
+    if (!both) break;
+    both = false;
+    minus = !minus;
+  }
+  out = best;
+  return big < FIX_DIFF_HI;
+}
+#endif
+
+// sqrt(acc) 2^-S / (12 h) as a double: acc = x 2^(128 - z), 1/4 <= x < 1, a
+// single-precision reciprocal root r0 of x, r = r0 (1 + e/2 + 3 e^2 / 8) with
+// e = 1 - x r0^2 (|e| < 2^-21), sqrt(x) = x r, rounded to 53 bits.
+ETD_HD double grad_of(U128 acc, const WenoInt& k) {
+  int z = 0;
+  if (acc.hi == 0) {
+    if (acc.lo == 0) return 0.0;
+    acc.hi = acc.lo;
+    acc.lo = 0;
+    z = 64;
+  }
+  int z1;
+  u64 M = normalise(acc, z1);
+  z += z1;
+  M >>= z & 1;
+  z &= ~1;
+  const unsigned mh = hi32(M);
+  const unsigned fb = (mh >> 31) ? 0x3f000000u | ((mh & 0x7fffffffu) >> 8) : 0x3e800000u | ((mh & 0x3fffffffu) >> 7);
+  float f, rf;
+#ifdef __CUDA_ARCH__
+  f = __uint_as_float(fb);
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
+  rf = fminf(rf, 1.9999998f);
+  const unsigned rb = __float_as_uint(rf);
+#else
+  memcpy(&f, &fb, 4);
+  rf = 1.0f / sqrtf(f);
+  if (rf > 1.9999998f) rf = 1.9999998f;
+  unsigned rb;
+  memcpy(&rb, &rf, 4);
+#endif
+  const unsigned r0 = (rb & 0x7fffffu) << 8 | 0x80000000u;  // (1, 2) 2^31
+  const i64 e = (i64)((1ull << 62) - mulhi_u(M, wide(r0, r0)));  // e 2^62
+  const int eh = (int)(e >> 16);
+  const i64 e1 = (e >> 1) + ((i64)eh * eh * 3 >> 33);
+  const i64 c = ((i64)r0 * (int)(e1 >> 16) + (i64)(wide(r0, (unsigned)e1 & 0xffffu) >> 16)) >> 14;
+  const u64 gx = mulhi_u(M, ((u64)r0 << 32) + (u64)c);  // sqrt(x) 2^63
+  const u64 bits = ((u64)(1085 - (z >> 1)) << 52) + ((gx + 512) >> 10);
+  double v;
+#ifdef __CUDA_ARCH__
+  v = __longlong_as_double((i64)bits);
+#else
+  memcpy(&v, &bits, 8);
+#endif
+  return v * k.scale;
+}
+
+}  // namespace etd
