@@ -598,11 +598,10 @@ __device__ __forceinline__ int sweep_level(uint8_t f) {
   return (f & F_V2) ? 0 : 1;
 }
 
-// Extension sweeps of the mixed variant: the same first-order upwind
-// iteration as the FP64 sweeps (three sweeps of K Jacobi passes over the
-// regions of levels >= 1, >= 2, 3; each sweep's result is the next one's
-// source), in FP32 arithmetic on FP32 copies of the fields, two passes per
-// grid barrier.  One pass at a region entry p is
+// Extension sweeps: first-order upwind iteration, three sweeps of K Jacobi
+// passes over the regions of levels >= 1, >= 2, 3 (each sweep's result is the
+// next one's source); in the mixed variant in FP32 arithmetic on FP32 copies
+// of the fields.  Two passes per grid barrier where that fits.  One pass at a region entry p is
 //   q'(p) = c0 q(p) + sum_d a_d q(u_d) + ds,   a_d = dtau |n_d| / h, c0 = 1 - sum_d a_d,
 // with u_d the upwind neighbour along d and ds = dtau s(p); nodes off the
 // region keep their values.  Two passes in one update from the values before
@@ -614,8 +613,8 @@ __device__ __forceinline__ int sweep_level(uint8_t f) {
 // nothing else.  A node met twice (u_de = u_ed; u_dd = p where the upwind
 // direction turns) keeps one term with the summed weight.  Each region entry
 // has a thread of its own when the region is at most one entry per thread;
-// larger regions take one pass per barrier.  The fields arrive in FP64 and the
-// extended u leaves in FP64.
+// larger regions take one pass per barrier (sweep_single).  The fields arrive
+// in FP64 and the extended u leaves in FP64.
 template <typename T>
 __device__ __forceinline__ T tfma(T x, T y, T z) {
   if constexpr (sizeof(T) == 4) return fmaf(x, y, z);
@@ -627,10 +626,82 @@ __device__ __forceinline__ T tabs(T x) {
   else return fabs(x);
 }
 
+// One sweep of K Jacobi passes over the first len entries of the sweep list,
+// one pass per grid barrier: X[0] holds q, the result is in X[K & 1]; dtau
+// and dth = dtau / h.  A thread keeps its first SW_CACHE entries (node, upwind
+// nodes, coefficients, own value, dtau s) in registers, so that a pass issues
+// its N neighbour loads at once and does N + 1 FMAs; entries past those (more
+// than SW_CACHE times the grid's threads) load them in every pass.  Measured
+// on regions of one to two entries per thread (4D, FP32, 83k nodes): 4.8 us a
+// pass with every entry loaded in every pass, 3.1 with the entries kept (3D,
+// 256^3: 3.55 and 2.34).
 template <int N, typename T>
-__device__ bool ext_sweeps_pair(const LsArgs& a, LsCtx& c, int n, long long cap, int K, double dtau, double dth,
+__device__ __noinline__ bool sweep_single(const LsArgs& a, LsCtx& c, long long len, long long cap, int K, T dtau, T dth,
+                                          T* const* X, const T* __restrict__ src) {
+  constexpr int SW_CACHE = 2;
+  const GridDev& g = a.g;
+  const long long gth = (long long)gridDim.x * blockDim.x, jt = dealt_tid();
+  int cp[SW_CACHE], cup[SW_CACHE][N];
+  T cq[SW_CACHE], cds[SW_CACHE], cc0[SW_CACHE], ca[SW_CACHE][N];
+  const auto load = [&](long long j, int& p, int* up, T& ds, T& c0, T* ad) {
+    const long long i = __ldcg(a.b.slist + j);
+    p = __ldcg(a.b.list + i);
+    ds = src ? dtau * __ldcg(src + p) : T(0);
+    int ix[N];
+    unpack<N>(__ldcg(a.b.lcoord + i), ix);
+    T asum = T(0);
+#pragma unroll
+    for (int d = 0; d < N; ++d) {
+      const double nd = __ldcg(a.b.nrm + d * cap + i);
+      up[d] = (int)nbr(g, p, ix, d, nd > 0.0 ? -1 : 1);
+      ad[d] = dth * tabs((T)nd);
+      asum += ad[d];
+    }
+    c0 = T(1) - asum;
+  };
+#pragma unroll
+  for (int r = 0; r < SW_CACHE; ++r) {
+    if (jt + r * gth >= len) continue;
+    load(jt + r * gth, cp[r], cup[r], cds[r], cc0[r], ca[r]);
+    cq[r] = __ldcg(X[0] + cp[r]);
+  }
+  for (int it = 0; it < K; ++it) {
+    const T* const qc = X[it & 1];
+    T* const qn = X[(it & 1) ^ 1];
+#pragma unroll
+    for (int r = 0; r < SW_CACHE; ++r) {
+      if (jt + r * gth >= len) continue;
+      T qu[N];
+#pragma unroll
+      for (int d = 0; d < N; ++d) qu[d] = __ldcg(qc + cup[r][d]);
+      T t = tfma(cc0[r], cq[r], cds[r]);
+#pragma unroll
+      for (int d = 0; d < N; ++d) t = tfma(ca[r][d], qu[d], t);
+      cq[r] = t;
+      qn[cp[r]] = t;
+    }
+    for (long long j = jt + SW_CACHE * gth; j < len; j += gth) {
+      int p, up[N];
+      T ds, c0, ad[N], qu[N];
+      load(j, p, up, ds, c0, ad);
+#pragma unroll
+      for (int d = 0; d < N; ++d) qu[d] = __ldcg(qc + up[d]);
+      T t = tfma(c0, __ldcg(qc + p), ds);
+#pragma unroll
+      for (int d = 0; d < N; ++d) t = tfma(ad[d], qu[d], t);
+      qn[p] = t;
+    }
+    if (!grid_barrier(a.st, c.bar, 57)) return false;
+  }
+  return true;
+}
+
+template <int N, typename T>
+__device__ bool ext_sweeps(const LsArgs& a, LsCtx& c, int n, long long cap, int K, double dtau, double dth,
                                const double* const* Q0) {
   constexpr int NTM = 1 + N + N * N;  // terms of a two-pass update
+  // 4D in FP64: 21 terms of an index and a weight spill the registers
+  constexpr bool PAIR = N <= 3 || sizeof(T) == 4;
   const GridDev& g = a.g;
   const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x, gth = (long long)gridDim.x * blockDim.x;
   const long long jt = dealt_tid();
@@ -667,7 +738,7 @@ __device__ bool ext_sweeps_pair(const LsArgs& a, LsCtx& c, int n, long long cap,
   // those of its upwind neighbours with their sweep levels, once.
   int p = 0, up[N], lev[N], tu[N][N];
   T c0 = T(0), ad[N], c0u[N], au[N][N];
-  if (jt < len0) {
+  if (PAIR && jt < len0) {
     const long long i = __ldcg(swl + jt);
     p = __ldcg(a.b.list + i);
     int ix[N];
@@ -707,7 +778,7 @@ __device__ bool ext_sweeps_pair(const LsArgs& a, LsCtx& c, int n, long long cap,
   int si = -1;  // field holding the source (the previous sweep's result)
   for (int sw = 0; sw < 3; ++sw) {
     const long long len = sw == 0 ? len0 : (sw == 1 ? sc2 + sc3 : sc3);
-    const bool two = K >= 2 && len <= gth;
+    const bool two = PAIR && len <= gth;
     T* const X[2] = {F[2 * sw], F[2 * sw + 1]};
     const T* const src = si < 0 ? nullptr : F[si];
     const bool has = two && jt < len;
@@ -773,37 +844,22 @@ __device__ bool ext_sweeps_pair(const LsArgs& a, LsCtx& c, int n, long long cap,
         cur ^= 1;
       }
     }
-    for (; it < K; ++it) {
-      const T* const qc = X[cur];
-      T* const qn = X[cur ^ 1];
-      if (has) {
-        T t = tfma(c0, cq, ds);
+    if (two) {
+      for (; it < K; ++it) {
+        if (has) {
+          const T* const qc = X[cur];
+          T t = tfma(c0, cq, ds);
 #pragma unroll
-        for (int d = 0; d < N; ++d) t = tfma(ad[d], __ldcg(qc + up[d]), t);
-        cq = t;
-        qn[p] = t;
-      } else if (!two) {
-        for (long long j = jt; j < len; j += gth) {
-          const long long i = __ldcg(swl + j);
-          const long long q = __ldcg(a.b.list + i);
-          int ix[N];
-          unpack<N>(__ldcg(a.b.lcoord + i), ix);
-          T asum = T(0), qu[N], aw[N];
-#pragma unroll
-          for (int d = 0; d < N; ++d) {
-            const double nd = __ldcg(a.b.nrm + d * cap + i);
-            qu[d] = __ldcg(qc + nbr(g, q, ix, d, nd > 0.0 ? -1 : 1));
-            aw[d] = dthf * tabs((T)nd);
-            asum += aw[d];
-          }
-          T t = tfma(T(1) - asum, __ldcg(qc + q), src ? dtf * __ldcg(src + q) : T(0));
-#pragma unroll
-          for (int d = 0; d < N; ++d) t = tfma(aw[d], qu[d], t);
-          qn[q] = t;
+          for (int d = 0; d < N; ++d) t = tfma(ad[d], __ldcg(qc + up[d]), t);
+          cq = t;
+          X[cur ^ 1][p] = t;
         }
+        if (!grid_barrier(a.st, c.bar, 57)) return false;
+        cur ^= 1;
       }
-      if (!grid_barrier(a.st, c.bar, 57)) return false;
-      cur ^= 1;
+    } else {
+      if (!sweep_single<N, T>(a, c, len, cap, K, dtf, dthf, X, src)) return false;
+      cur = K & 1;
     }
     si = 2 * sw + cur;
   }
@@ -812,109 +868,6 @@ __device__ bool ext_sweeps_pair(const LsArgs& a, LsCtx& c, int n, long long cap,
   for (long long i = gtid; i < n; i += gth) {
     const long long p = __ldcg(a.b.list + i);
     a.u[p] = sweep_level(__ldcg(a.b.lflag + i)) == 3 ? (double)__ldcg(F[si] + p) : __ldcg(Q0[2] + p);
-  }
-  return true;
-}
-
-// Extension sweeps in FP64 (the plain and the reference arithmetic): three
-// sweeps of K Jacobi passes, one pass per grid barrier (see the caller for
-// the update).  The extended u goes to the caller's array on the work list.
-template <int N>
-__device__ bool ext_sweeps_f64(const LsArgs& a, LsCtx& c, int n, long long cap, int K, double dtau, double dth,
-                               double* const* UNN, double* const* UN, double* const* U) {
-  const GridDev& g = a.g;
-  const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x, gth = (long long)gridDim.x * blockDim.x;
-  double* const* bufs[3] = {UNN, UN, U};
-  const double* src = nullptr;
-  constexpr int SW_CACHE = 2;
-  const int* const swl = a.b.slist;
-  const int sc1 = __ldcg(a.b.sw + 1), sc2 = __ldcg(a.b.sw + 2), sc3 = __ldcg(a.b.sw + 3);
-  const long long jt = dealt_tid();
-  for (int sw = 0; sw < 3; ++sw) {
-    double* const* B = bufs[sw];
-    const long long len = sw == 0 ? sc1 + sc2 + sc3 : (sw == 1 ? sc2 + sc3 : sc3);
-    for (long long i = gtid; i < n; i += gth) {
-      const long long p = __ldcg(a.b.list + i);
-      B[1][p] = __ldcg(B[0] + p);
-    }
-    int cp[SW_CACHE], cup[SW_CACHE][N];
-    bool creg[SW_CACHE];
-    double cq[SW_CACHE], cds[SW_CACHE], cc0[SW_CACHE], ca[SW_CACHE][N];
-#pragma unroll
-    for (int r = 0; r < SW_CACHE; ++r) {
-      const long long j = jt + r * gth;
-      creg[r] = j < len;
-      cp[r] = 0;
-      cq[r] = cds[r] = cc0[r] = 0.0;
-#pragma unroll
-      for (int d = 0; d < N; ++d) {
-        cup[r][d] = 0;
-        ca[r][d] = 0.0;
-      }
-      if (creg[r]) {
-        const long long i = __ldcg(swl + j);
-        const long long p = __ldcg(a.b.list + i);
-        cp[r] = (int)p;
-        cq[r] = __ldcg(B[0] + p);
-        cds[r] = src ? dtau * __ldcg(src + p) : 0.0;
-        int ix[N];
-        unpack<N>(a.b.lcoord[i], ix);
-        double asum = 0.0;
-#pragma unroll
-        for (int d = 0; d < N; ++d) {
-          const double nd = __ldcg(a.b.nrm + d * cap + i);
-          cup[r][d] = (int)nbr(g, p, ix, d, nd > 0.0 ? -1 : 1);
-          ca[r][d] = dth * fabs(nd);
-          asum += ca[r][d];
-        }
-        cc0[r] = 1.0 - asum;
-      }
-    }
-    if (!grid_barrier(a.st, c.bar, 53)) return false;
-    int cur = 0;
-    for (int it = 0; it < K; ++it) {
-      const double* qc = B[cur];
-      double* qn = B[cur ^ 1];
-#pragma unroll
-      for (int r = 0; r < SW_CACHE; ++r) {
-        if (!creg[r]) continue;
-        double qu[N];
-#pragma unroll
-        for (int d = 0; d < N; ++d) qu[d] = __ldcg(qc + cup[r][d]);
-        double t = fma(cc0[r], cq[r], cds[r]);
-#pragma unroll
-        for (int d = 0; d < N; ++d) t = fma(ca[r][d], qu[d], t);
-        cq[r] = t;
-        qn[cp[r]] = t;
-      }
-      for (long long j = jt + SW_CACHE * gth; j < len; j += gth) {
-        const long long i = __ldcg(swl + j);
-        const long long p = __ldcg(a.b.list + i);
-        int ix[N];
-        unpack<N>(a.b.lcoord[i], ix);
-        double asum = 0.0, qu[N], ad[N];
-#pragma unroll
-        for (int d = 0; d < N; ++d) {
-          const double nd = __ldcg(a.b.nrm + d * cap + i);
-          qu[d] = __ldcg(qc + nbr(g, p, ix, d, nd > 0.0 ? -1 : 1));
-          ad[d] = dth * fabs(nd);
-          asum += ad[d];
-        }
-        const double ds = src ? dtau * __ldcg(src + p) : 0.0;
-        double t = fma(1.0 - asum, __ldcg(qc + p), ds);
-#pragma unroll
-        for (int d = 0; d < N; ++d) t = fma(ad[d], qu[d], t);
-        qn[p] = t;
-      }
-      if (!grid_barrier(a.st, c.bar, 53)) return false;
-      cur ^= 1;
-    }
-    src = B[cur];
-  }
-  // extended u back to the caller's array on the work list
-  for (long long i = gtid; i < n; i += gth) {
-    const long long p = __ldcg(a.b.list + i);
-    a.u[p] = __ldcg(src + p);
   }
   return true;
 }
@@ -1318,21 +1271,15 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
   // first-order upwind step
   //   q' = q - dtau (sum_d n_d D_d q - s),  D_d backward where n_d > 0,
   // is used in the rearranged form q' = c0 q + sum_d a_d q(up_d) + dtau s,
-  // a_d = dtau |n_d| / h, c0 = 1 - sum_d a_d (equal up to rounding).  Each
-  // thread keeps its first SW_CACHE region entries (node, upwind nodes,
-  // coefficients, own value, dtau s) in registers, so a pass issues its N
-  // neighbour loads at once and does N + 1 FMAs.
+  // a_d = dtau |n_d| / h, c0 = 1 - sum_d a_d (equal up to rounding).
   const int K = (int)ceil(12.0 * sqrt((double)N));
   const double dtau = h / (2.0 * sqrt((double)N));
   const double dth = dtau * inv_h;
   {
     const double* const Q0[3] = {UNN[0], UN[0], U[0]};
-    const long long len0 = (long long)__ldcg(a.b.sw + 1) + __ldcg(a.b.sw + 2) + __ldcg(a.b.sw + 3);
     if (a.mixed) {
-      if (!ext_sweeps_pair<N, float>(a, c, n, cap, K, dtau, dth, Q0)) return;
-    } else if (N <= 3 && len0 <= gth) {
-      if (!ext_sweeps_pair<N, double>(a, c, n, cap, K, dtau, dth, Q0)) return;
-    } else if (!ext_sweeps_f64<N>(a, c, n, cap, K, dtau, dth, UNN, UN, U)) {
+      if (!ext_sweeps<N, float>(a, c, n, cap, K, dtau, dth, Q0)) return;
+    } else if (!ext_sweeps<N, double>(a, c, n, cap, K, dtau, dth, Q0)) {
       return;
     }
   }
