@@ -663,10 +663,12 @@ __device__ __noinline__ QuadSums quad_stencil(const float* __restrict__ X, float
 // vectors).  Measured per launch with the earlier two-pass kernel at 256^3 /
 // 512^3 (10 / 20 vectors): 5 in flight 1.378 / 14.11 ms, 8 1.376 / 14.01,
 // 10 1.342 / 13.51, 16 1.390 / 13.72.  Writes y (compact, FP64) and its FP32
-// grid copy (0 at the group's other nodes), and, for the last substep, y
-// into ufin at the computational points (the kernel then skips its
-// write-back); returns this thread's sum of the squares of the FP32 copy
-// (the controller's scale).  Inlined into the kernel: 1.59 against 1.80 ms
+// grid copy (0 at the group's other nodes) and returns this thread's sum of
+// the squares of the FP32 copy (the controller's scale); or, for the last
+// substep, writes y into ufin at the computational points and nothing else,
+// returning infinity if a value is not finite
+// (the kernel then skips its write-back; y, its copy and its norm are read by
+// a further substep only, and the next call writes them anew).  Inlined into the kernel: 1.59 against 1.80 ms
 // at 512^3 out of line.
 static __device__ __forceinline__ double quad_combination(const float* __restrict__ chi,
                                                           const float* __restrict__ clo, int m, double tau,
@@ -678,6 +680,8 @@ static __device__ __forceinline__ double quad_combination(const float* __restric
                                                           int nq, long long gtid, long long gth) {
   Acc<float> yn;  // |y|^2 of the FP32 copy: the controller's scale only
   const double h2 = 0.5 * tau * tau;
+  unsigned top = 0;  // last substep: largest leading word of |y|, for the finiteness check
+  const bool u16 = ufin != nullptr && (reinterpret_cast<uintptr_t>(ufin) & 15u) == 0;
   quad_loop(qidx, qk, nq, gtid, gth, [&](long long p4, int k0, bool full, long long pn4) {
     if (pn4 >= 0 && (pn4 & 31) == 0)  // a lane per 128-byte line
       for (int i = 0; i < m; ++i) prefetch_l2(V + (long long)i * vs + pn4);
@@ -696,6 +700,19 @@ static __device__ __forceinline__ double quad_combination(const float* __restric
     const float4 w2 = W2g ? ld4(W2g + p4) : make_float4(0.f, 0.f, 0.f, 0.f);
     const float sl[4] = {s0, s1, s2, s3}, el[4] = {e0, e1, e2, e3};
     const float w1l[4] = {w1.x, w1.y, w1.z, w1.w}, w2l[4] = {w2.x, w2.y, w2.z, w2.w};
+    if (full && u16) {
+      double y[4];
+#pragma unroll
+      for (int l = 0; l < 4; ++l) {
+        y[l] = fma(tau, to_f64(w1l[l]), __ldcg(Yc + k0 + l)) + (to_f64(sl[l]) + to_f64(el[l]));
+        if (W2g) y[l] = fma(h2, to_f64(w2l[l]), y[l]);
+      }
+#pragma unroll
+      for (int l = 0; l < 4; ++l) top = max(top, (unsigned)__double2hiint(y[l]) & 0x7fffffffu);
+      __stcg(reinterpret_cast<double2*>(ufin + p4), make_double2(y[0], y[1]));
+      __stcg(reinterpret_cast<double2*>(ufin + p4 + 2), make_double2(y[2], y[3]));
+      return;
+    }
     float yo[4];
     int rank = 0;
 #pragma unroll
@@ -706,13 +723,18 @@ static __device__ __forceinline__ double quad_combination(const float* __restric
       ++rank;
       double y = fma(tau, to_f64(w1l[l]), __ldcg(Yc + k)) + (to_f64(sl[l]) + to_f64(el[l]));
       if (W2g) y = fma(h2, to_f64(w2l[l]), y);
+      if (ufin != nullptr) {
+        top = max(top, (unsigned)__double2hiint(y) & 0x7fffffffu);
+        ufin[p4 + l] = y;
+        continue;
+      }
       Yc[k] = y;
-      if (ufin != nullptr) ufin[p4 + l] = y;
       yo[l] = to_f32_rn(y);
       yn.add(yo[l], yo[l]);
     }
-    st4(Yg + p4, make_float4(yo[0], yo[1], yo[2], yo[3]));
+    if (ufin == nullptr) st4(Yg + p4, make_float4(yo[0], yo[1], yo[2], yo[3]));
   });
+  if (ufin != nullptr) return top >= 0x7ff00000u ? (double)INFINITY : 0.0;
   return yn.value();
 }
 
