@@ -414,11 +414,6 @@ struct AccG {
   __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
 
-// groups per thread and iteration in quad_pass_1 (two measured slower at
-// 512^3: 322 against 262 us per pass; the registers, not the index loads,
-// bound the loads in flight)
-constexpr int QP_U = 1;
-
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // Top bit of a group's list entry qk: its 4 nodes are computational and
@@ -472,7 +467,10 @@ __device__ __forceinline__ void quad_loop(const int* __restrict__ qidx, const in
 // AccG sums), from which alpha_j and beta_{j+1} follow without another
 // pass.  Two vectors are read (each with its stencil) and two written.  A
 // V_j value is formed by the same two roundings wherever it is formed, so
-// Z_j is A applied to the stored V_j.  Inlined into the kernel: out of line
+// Z_j is A applied to the stored V_j.  The end values from the neighbouring
+// lanes and no class or diagonal work in warps of full groups took the pass
+// from 249 to 203 us at 512^3 (47M points; the same loads and stores without
+// the arithmetic take 152 us).  Inlined into the kernel: out of line
 // its 20-odd register arguments and the saves around the call cost the
 // 768-thread kernel 8% per pass at 512^3 (4.93 against 5.34 ms for 19 passes).
 template <int N>
@@ -482,57 +480,55 @@ __device__ __forceinline__ QuadSums quad_pass_1(const float* __restrict__ Wp, co
                                                 const float* __restrict__ diagf, const int* __restrict__ qidx,
                                                 const int* __restrict__ qk, int nq, const GridDev& g, float cfac,
                                                 float bc, float dint, long long gtid, long long gth) {
-  constexpr int U = QP_U;
   long long st[N > 1 ? N - 1 : 1];
 #pragma unroll
   for (int d = 0; d < N - 1; ++d) st[d] = g.stride[d];
   AccG d1, d2, d3;
   const auto vnew = [c1, c2](float w, float v) { return __fmaf_rn(c2, v, __fmul_rn(c1, w)); };
-  // this iteration's groups q + u gth, the next iteration's, and (loaded
-  // here) the one after: an iteration's data loads never wait on its index
-  // loads, and the next iteration's lines are prefetched into L2
-  int pc[U], kc[U], pn[U], kn[U];
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const long long q0 = gtid + u * gth, q1 = gtid + (U + u) * gth;
-    pc[u] = q0 < nq ? __ldg(qidx + q0) : -1;
-    kc[u] = q0 < nq ? __ldg(qk + q0) : 0;
-    pn[u] = q1 < nq ? __ldg(qidx + q1) : -1;
-    kn[u] = q1 < nq ? __ldg(qk + q1) : 0;
-  }
-  for (long long q = gtid; q < nq; q += U * gth) {
-    int pf[U], kf[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const long long q2 = q + (2 * U + u) * gth;
-      pf[u] = q2 < nq ? __ldg(qidx + q2) : -1;
-      kf[u] = q2 < nq ? __ldg(qk + q2) : 0;
-      if (pn[u] >= 0 && (pn[u] & 7) == 0) {
-        // the next groups' own lines and those of their upper neighbours
-        // along the first axis (the only ones no earlier group brought in),
-        // by the lane whose group starts a 128-byte line of the FP32 vectors
-        const long long pn4 = (long long)pn[u] << 2;
-        prefetch_l2(Wp + pn4);
-        prefetch_l2(Vp + pn4);
-        prefetch_l2(Wp + pn4 + st[0]);
-        prefetch_l2(Vp + pn4 + st[0]);
-      }
+  // cfac (bc s - D x) + c3 v, the roundings fixed so that both kinds of warp
+  // give the same bits
+  const auto unew = [cfac, bc, c3](float s, float D, float x, float v) {
+    return __fmaf_rn(cfac, __fmaf_rn(bc, s, -__fmul_rn(D, x)), __fmul_rn(c3, v));
+  };
+  const int lane = threadIdx.x & 31;
+  // this iteration's group, the next one's, and (loaded here) the one after:
+  // an iteration's data loads never wait on its index loads, and the next
+  // iteration's lines are prefetched into L2.  Whole warps: the values at a
+  // group's ends are the neighbouring lanes' where those hold the adjacent
+  // groups (most do), and a warp of full groups takes no class or diagonal.
+  int pc = gtid < nq ? __ldg(qidx + gtid) : -1, kc = gtid < nq ? __ldg(qk + gtid) : QK_FULL;
+  int pn = gtid + gth < nq ? __ldg(qidx + gtid + gth) : -1, kn = gtid + gth < nq ? __ldg(qk + gtid + gth) : QK_FULL;
+  for (long long q = gtid; q - lane < nq; q += gth) {
+    const long long q2 = q + 2 * gth;
+    const int pf = q2 < nq ? __ldg(qidx + q2) : -1, kf = q2 < nq ? __ldg(qk + q2) : QK_FULL;
+    if (pn >= 0 && (pn & 7) == 0) {
+      // the next groups' own lines and those of their upper neighbours
+      // along the first axis (the only ones no earlier group brought in),
+      // by the lane whose group starts a 128-byte line of the FP32 vectors
+      const long long pn4 = (long long)pn << 2;
+      prefetch_l2(Wp + pn4);
+      prefetch_l2(Vp + pn4);
+      prefetch_l2(Wp + pn4 + st[0]);
+      prefetch_l2(Vp + pn4 + st[0]);
     }
-    float4 wc[U], vc[U], sacc[U], dg[U];
-    float wl[U], wr[U], vl[U], vr[U];
-    unsigned kw[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (pc[u] < 0) continue;
-      const long long p4 = (long long)pc[u] << 2;
-      const int k0 = kc[u] & QK_INDEX;
-      wc[u] = ld4(Wp + p4);
-      vc[u] = ld4(Vp + p4);
-      wl[u] = __ldcg(Wp + p4 - 1);
-      wr[u] = __ldcg(Wp + p4 + 4);
-      vl[u] = __ldcg(Vp + p4 - 1);
-      vr[u] = __ldcg(Vp + p4 + 4);
-      float4 sa = make_float4(-0.f, -0.f, -0.f, -0.f);  // as stencil()
+    const int ql = __shfl_up_sync(0xffffffffu, pc, 1), qr = __shfl_down_sync(0xffffffffu, pc, 1);
+    const bool all_full = __all_sync(0xffffffffu, kc < 0);
+    const bool act = pc >= 0;
+    const long long p4 = act ? (long long)pc << 2 : 0ll;
+    float4 wc = make_float4(0.f, 0.f, 0.f, 0.f), vc = wc, sa = make_float4(-0.f, -0.f, -0.f, -0.f);  // as stencil()
+    float wl = 0.f, wr = 0.f, vl = 0.f, vr = 0.f;
+    const bool nl = lane == 0 || ql != pc - 1, nr = lane == 31 || qr != pc + 1;
+    if (act) {
+      wc = ld4(Wp + p4);
+      vc = ld4(Vp + p4);
+      if (nl) {
+        wl = __ldcg(Wp + p4 - 1);
+        vl = __ldcg(Vp + p4 - 1);
+      }
+      if (nr) {
+        wr = __ldcg(Wp + p4 + 4);
+        vr = __ldcg(Vp + p4 + 4);
+      }
 #pragma unroll
       for (int d = 0; d < N - 1; ++d) {
         const float4 wm = ld4(Wp + p4 - st[d]), wq = ld4(Wp + p4 + st[d]);
@@ -542,32 +538,42 @@ __device__ __forceinline__ QuadSums quad_pass_1(const float* __restrict__ Wp, co
         sa.z += vnew(wm.z, vm.z) + vnew(wq.z, vq.z);
         sa.w += vnew(wm.w, vm.w) + vnew(wq.w, vq.w);
       }
-      sacc[u] = sa;
-      kw[u] = kc[u] < 0 ? QK_FULL_KIND : __ldg(reinterpret_cast<const unsigned*>(kind + p4));
-      dg[u] = kc[u] < 0 ? make_float4(dint, dint, dint, dint)
-                        : make_float4(__ldg(diagf + k0), __ldg(diagf + k0 + 1), __ldg(diagf + k0 + 2),
-                                      __ldg(diagf + k0 + 3));
     }
+    // V_j along the last axis: the group's left neighbour, its 4 nodes, its right neighbour
+    float x[6];
+    x[1] = vnew(wc.x, vc.x);
+    x[2] = vnew(wc.y, vc.y);
+    x[3] = vnew(wc.z, vc.z);
+    x[4] = vnew(wc.w, vc.w);
+    x[0] = __shfl_up_sync(0xffffffffu, x[4], 1);
+    x[5] = __shfl_down_sync(0xffffffffu, x[1], 1);
+    if (nl) x[0] = vnew(wl, vl);
+    if (nr) x[5] = vnew(wr, vr);
+    const float so[4] = {sa.x, sa.y, sa.z, sa.w};
+    const float vp[4] = {vc.x, vc.y, vc.z, vc.w};
+    float z[4];
+    if (all_full) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (pc[u] < 0) continue;
-      const long long p4 = (long long)pc[u] << 2;
-      // V_j along the last axis: the group's left neighbour, its 4 nodes, its right neighbour
-      const float x[6] = {vnew(wl[u], vl[u]), vnew(wc[u].x, vc[u].x), vnew(wc[u].y, vc[u].y),
-                          vnew(wc[u].z, vc[u].z), vnew(wc[u].w, vc[u].w), vnew(wr[u], vr[u])};
-      const float so[4] = {sacc[u].x, sacc[u].y, sacc[u].z, sacc[u].w};
-      const float vp[4] = {vc[u].x, vc[u].y, vc[u].z, vc[u].w};
-      float z[4];
+      for (int l = 0; l < 4; ++l)  // as stencil(): the last axis is added last
+        z[l] = unew(so[l] + (x[l] + x[l + 2]), dint, x[l + 1], vp[l]);
+    } else {
+      const int k0 = kc & QK_INDEX;
+      unsigned kw = QK_FULL_KIND;
+      float4 dg = make_float4(dint, dint, dint, dint);
+      if (kc >= 0) {
+        kw = __ldg(reinterpret_cast<const unsigned*>(kind + p4));
+        dg = make_float4(__ldg(diagf + k0), __ldg(diagf + k0 + 1), __ldg(diagf + k0 + 2), __ldg(diagf + k0 + 3));
+      }
       int rank = 0;
 #pragma unroll
       for (int l = 0; l < 4; ++l) {
-        const bool comp = ((kw[u] >> (8 * l)) & 3u) == K_COMP;
-        const float D = rank == 0 ? dg[u].x : rank == 1 ? dg[u].y : rank == 2 ? dg[u].z : dg[u].w;
-        // as stencil(): the last axis is added last
-        const float az = cfac * (bc * (so[l] + (x[l] + x[l + 2])) - D * x[l + 1]);
-        z[l] = comp ? az + c3 * vp[l] : 0.f;
+        const bool comp = ((kw >> (8 * l)) & 3u) == K_COMP;
+        const float D = rank == 0 ? dg.x : rank == 1 ? dg.y : rank == 2 ? dg.z : dg.w;
+        z[l] = comp ? unew(so[l] + (x[l] + x[l + 2]), D, x[l + 1], vp[l]) : 0.f;
         rank += comp ? 1 : 0;
       }
+    }
+    if (act) {
       st4(Vj + p4, make_float4(x[1], x[2], x[3], x[4]));
       st4(Wn + p4, make_float4(z[0], z[1], z[2], z[3]));
       const float xv[4] = {x[1], x[2], x[3], x[4]};
@@ -575,13 +581,10 @@ __device__ __forceinline__ QuadSums quad_pass_1(const float* __restrict__ Wp, co
       d2.add4(z, xv);
       d3.add4(z, z);
     }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      pc[u] = pn[u];
-      kc[u] = kn[u];
-      pn[u] = pf[u];
-      kn[u] = kf[u];
-    }
+    pc = pn;
+    kc = kn;
+    pn = pf;
+    kn = kf;
   }
   return QuadSums{d1.value(), d2.value(), d3.value()};
 }
@@ -749,7 +752,11 @@ __device__ __forceinline__ bool quad_full(const SpeciesDev<T>& S, int ncomp, int
 // Builds the quad list from the sorted list of computational points: each
 // warp takes a contiguous range of list indices (ranges in block, then warp
 // order); a list index starts a group when its group differs from the
-// previous index's.  Counts per warp, one grid barrier for the per-block
+// previous index's.  Within each range the full groups (QK_FULL) come first, in
+// order, and the others last, from the range's end down: nearly every warp of a pass then holds full
+// groups only, while a range's groups stay close enough to share L2 lines
+// (two separate lists would fetch the others' neighbours from DRAM again).
+// Counts per warp, one grid barrier for the per-block
 // totals, then ordered writes at the warp's offset (warp ballots, no block
 // barrier in the loop), then a grid barrier: the passes read entries other
 // CTAs wrote.  Eight 32-index loads in flight per warp.  Returns false if
@@ -802,6 +809,7 @@ __device__ bool build_quads(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int n
   __syncthreads();
   int base = c.qoff;
   for (int w = 0; w < wid; ++w) base += s_wc[w];
+  int bpart = base + cnt - 1;  // the range's other groups, from its end down
   const unsigned below = (1u << lane) - 1u;
   for (long long kb = kw0; kb < kw1; kb += 32 * QU) {
     int q[QU], qp[QU];
@@ -814,14 +822,16 @@ __device__ bool build_quads(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int n
 #pragma unroll
     for (int u = 0; u < QU; ++u) {
       const bool head = q[u] >= 0 && qp[u] != q[u];
-      const unsigned bal = __ballot_sync(0xffffffffu, head);
+      const long long k = kb + u * 32 + lane;
+      const bool full = head && quad_full<T, N>(S, ncomp, q[u], k);
+      const unsigned bf = __ballot_sync(0xffffffffu, full), bp = __ballot_sync(0xffffffffu, head && !full);
       if (head) {
-        const int pos = base + __popc(bal & below);
-        const long long k = kb + u * 32 + lane;
+        const int pos = full ? base + __popc(bf & below) : bpart - __popc(bp & below);
         S.qidx[pos] = q[u];
-        S.qk[pos] = (int)k | (quad_full<T, N>(S, ncomp, q[u], k) ? QK_FULL : 0);
+        S.qk[pos] = (int)k | (full ? QK_FULL : 0);
       }
-      base += __popc(bal);
+      base += __popc(bf);
+      bpart -= __popc(bp);
     }
   }
   return grid_barrier(a.st, bar, 26);
