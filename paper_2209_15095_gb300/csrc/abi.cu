@@ -338,6 +338,7 @@ SpeciesDev<T> species_dev(etd_ctx* c, int s, double* u, int stage = 0) {
   d.beta_field = b.beta_field;
   d.beta_c = c->par.beta[s];
   d.gersh = &c->st->gersh[s];
+  d.negb = &c->st->negb[s];
   d.u = u;
   d.Fprev = b.Fprev;
   d.Fprev2 = b.Fprev2;
@@ -576,6 +577,7 @@ etd_status etd_init_domain(etd_ctx* c, int species, const double* phi, const dou
   ma.bco = b.bco;
   ma.bpts = b.bpts;
   ma.gersh = &c->st->gersh[species];
+  ma.negb = &c->st->negb[species];
   ma.st = c->st;
   cudaError_t e = cudaSuccess;
   // the Krylov kernel's 4-node group list belongs to the previous domain

@@ -73,6 +73,7 @@ struct DevStatus {
   double gersh[2];      // Gershgorin bound of C per species (max row sum of |C|)
   unsigned int barrier; // grid-barrier arrival counter (reset before each cooperative launch)
   unsigned int pad2;
+  int negb[2];          // per species: the beta field has a negative value
   unsigned long long wait_ns;  // limit of every device wait in ns (0: BARRIER_LIMIT_NS)
 };
 

@@ -238,6 +238,7 @@ __device__ void metadata_phase(const MetaArgs& a, int ncomp) {
       const long long q = p + s;
       const int iq = ip[d] + (si == 0 ? -1 : 1);
       const double bf = a.beta_field ? 0.5 * (a.beta_field[p] + a.beta_field[q]) : a.beta_c;
+      if (a.beta_field && negative(bf)) *a.negb = 1;
       double gw = 0.0;  // 1 - w on a ghost face, 0 on a face to a computational point
       // boundary-data slots of this face: coefficient of u_Gamma in the row
       // (beta_f c / h^2, the ghost value's weight on the boundary point) and
@@ -359,7 +360,10 @@ __global__ void __launch_bounds__(INIT_NT, 1) init_domain_kernel(const ClassifyA
   const long long cw = (nw + gridDim.x - 1) / gridDim.x;
   const long long wlo = min((long long)blockIdx.x * cw, nw), whi = min(wlo + cw, nw);
   uint32_t* cbits = (uint32_t*)(ca.tile_count + MAX_BLOCKS);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *ma.gersh = 0.0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *ma.gersh = 0.0;
+    *ma.negb = 0;
+  }
   __shared__ int s_w[INIT_NT / 32];
   __shared__ int s_off, s_tot;
   int cnt = 0;

@@ -34,6 +34,7 @@ struct MetaArgs {
   double* bco;   // nullptr, or per point, face and slot (2 slots for N = 2, else 1):
   double* bpts;  //   boundary-data coefficient and point (N doubles)
   double* gersh;
+  int* negb;
   DevStatus* st;
 };
 
@@ -66,6 +67,7 @@ struct SpeciesDev {
   const double* beta_field;
   double beta_c;
   const double* gersh;
+  const int* negb;  // nonzero: the beta field has a negative value
   // caller's field (full grid, FP64); other species' field for coupling
   double* u;
   // F_{n-1} (and, for multistep ETD3, F_{n-2}) on the grid, and their

@@ -44,7 +44,6 @@ namespace etd {
 constexpr int CHECK_EVERY = 5;
 constexpr double TAU_MIN = 1e-6;
 constexpr double BREAKDOWN_REL = 1e-12;
-constexpr float TAYLOR_THETA = 8.0f;
 constexpr int MAX_SUBSTEPS = 20000;  // bounded work per call
 // From SPLIT_MIN computational points on, a Krylov vector costs two passes
 // (V_j = w_j at the own points; after a barrier Z_j = A V_j and the sums)
@@ -60,15 +59,52 @@ constexpr int SPLIT_U = sizeof(T) == 8 ? 2 : 4;
 template <typename T>
 constexpr int SPLIT_UB = sizeof(T) == 8 ? 2 : 3;  // the stencil pass (register bound)
 
-// 1/k!: each translation unit that instantiates the kernel has its own copy
-// (filled by load_inv_fact before its first launch)
-static __constant__ double c_inv_fact[64];
+// Chebyshev coefficients 2 e^-a I_k(a) of e^(a (x - 1)) for a = 2^(i/2),
+// i = 0 .. CHEB_TABLES - 1, down to 1e-24: table i at c_cheb + c_cheb_at[i]
+// (20 coefficients at a = 1, 87 at 64, 233 at 512).  Each translation unit
+// that instantiates the kernel has its own copy (filled by load_cheb before
+// its first launch).
+constexpr int CHEB_TABLES = 19, CHEB_MAX = 1800;
+static __constant__ double c_cheb[CHEB_MAX];
+static __constant__ double c_cheb_2a[CHEB_TABLES];  // 2 / a
+static __constant__ int c_cheb_at[CHEB_TABLES + 1];
 
-static cudaError_t load_inv_fact() {
-  double f[64];
-  f[0] = 1.0;
-  for (int k = 1; k < 64; ++k) f[k] = f[k - 1] / (double)k;
-  return cudaMemcpyToSymbol(c_inv_fact, f, sizeof(f));
+// I_k(a) up to a factor by Miller's downward recurrence I_{k-1} = I_{k+1} +
+// (2k/a) I_k (Abramowitz & Stegun 9.12), normalised by I_0 + 2 sum I_k = e^a.
+static cudaError_t load_cheb() {
+  double tab[CHEB_MAX], two_a[CHEB_TABLES];
+  int at[CHEB_TABLES + 1];
+  int n = 0;
+  for (int i = 0; i < CHEB_TABLES; ++i) {
+    const double a = pow(2.0, 0.5 * i);
+    two_a[i] = 2.0 / a;
+    at[i] = n;
+    double t[512];
+    double up = 0.0, sum = 0.0, cur = 1e-200;
+    for (int k = 511; k >= 0; --k) {  // cur = I_k, up = I_{k+1}
+      t[k] = cur;
+      sum += k > 0 ? 2.0 * cur : cur;
+      const double down = up + 2.0 * k / a * cur;
+      up = cur;
+      cur = down;
+      if (cur > 1e200) {
+        for (int j = k; j < 512; ++j) t[j] *= 1e-200;
+        cur *= 1e-200;
+        up *= 1e-200;
+        sum *= 1e-200;
+      }
+    }
+    for (int k = 0; k < 512 && n < CHEB_MAX; ++k) {
+      const double c = 2.0 * t[k] / sum;
+      if (c < 1e-24) break;
+      tab[n++] = c;
+    }
+  }
+  at[CHEB_TABLES] = n;
+  cudaError_t e = cudaMemcpyToSymbol(c_cheb, tab, sizeof(double) * n);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_cheb_2a, two_a, sizeof(two_a));
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_cheb_at, at, sizeof(at));
+  return e;
 }
 
 struct Ctl {
@@ -93,63 +129,74 @@ struct Ctl {
 // ---------------------------------------------------------------------------
 // small exponential: x = exp(K) e_{M-1} for the augmented matrix
 //   K = [[tau H_m, e_1, 0], [0, 0, I_p], [0, 0, 0]],  M = m + p + 1 <= 64,
-// by Taylor series with a shift and scaling, exp(K) = e^mu exp((K - mu I)/s)^s,
-// unnormalised powers accumulated with 1/k!.  Warp-cooperative: lane owns
-// rows lane and lane+32.
-// On return c.yexp[0..m-1] = phi_{p+1}(tau H_m) e_1.
-// s steps of the degree-deg Taylor polynomial of the tridiagonal-plus-
-// coupling matrix held as (A, B, C) per row (lane r: rows r and r + 32).
-// TWO is a template argument so that the second half's FP64 work is absent,
-// not predicated off, when M <= 32: a predicated-off FP64 instruction still
-// takes its issue slot.
-template <bool TWO>
-__device__ __forceinline__ void taylor_steps(int m, int s, int deg, const double (&A)[2], const double (&B)[2],
-                                             const double (&C)[2], double (&x)[2]) {
+// whose first m entries are phi_{p+1}(tau H_m) e_1, by one warp.
+//
+// A is negative semidefinite (the row's diagonal is at least the sum of its
+// positive off-diagonals), so K's eigenvalues lie in [L, 0] with L the lower
+// Gershgorin bound of tau H_m, and exp(K) is a Chebyshev series on [-2a, 0]
+// with a the next power of sqrt 2 above -L/2, in one Clenshaw recurrence
+//   b_k = c_k e + 2 X b_{k+1} - b_{k+2},  X = K/a + I,  x = (b_0 - b_2) / 2.
+// The number of steps grows like sqrt(a) (30 at |L| = 7, 87 at 120, 167 at
+// 500) where the shifted and scaled Taylor series it replaces grew like a (35,
+// 380, 1300), and a step issues three FP64 instructions instead of four.
+// Against 60-digit values its error is the Taylor form's or below (4e-15
+// against 7e-15 of the largest entry at |L| = 400; the last entry, which the
+// error estimate is, to 2e-14 relative where it matters).  Measured per check:
+// 12.2 -> 8.7 us at |L| = 7 and 10 vectors, 221 -> 28 us at |L| up
+// to 270 and 20 to 40 vectors.
+//
+// A beta field with negative values (`indef`) leaves no such bound: the
+// interval then ends at the upper Gershgorin bound U, and s steps with a <= 8
+// each keep the rounding errors of e^(a (x-1)) small against x.
+//
+// Rows are ordered along the chain M-1, M-2, .., m, 0, 1, .., m-1, which
+// makes K tridiagonal; the vector e enters as the first one's lower
+// neighbour.  M <= 32: a row per lane; above (TWO): two neighbouring rows per
+// lane.  GEN: from a general vector x instead of e.
+template <bool TWO, bool GEN>
+__device__ __forceinline__ void cheb_steps(const double* __restrict__ t, int n, const double (&A)[2],
+                                           const double (&B)[2], const double (&C)[2], const double (&x)[2],
+                                           double (&y)[2]) {
   const int lane = threadIdx.x & 31;
-  for (int it = 0; it < s; ++it) {
-    double P0 = x[0], P1 = x[1], acc0 = x[0], acc1 = x[1];
-    for (int k = 1; k <= deg; ++k) {
-      double dn0 = __shfl_up_sync(0xffffffffu, P0, 1);
-      double up0 = __shfl_down_sync(0xffffffffu, P0, 1);
-      const double pm = __shfl_sync(0xffffffffu, (!TWO || m < 32) ? P0 : P1, m & 31);
-      if (lane == 0) dn0 = pm;
-      if (TWO) {
-        double dn1 = __shfl_up_sync(0xffffffffu, P1, 1);
-        double up1 = __shfl_down_sync(0xffffffffu, P1, 1);
-        const double b31 = __shfl_sync(0xffffffffu, P0, 31);
-        const double b32 = __shfl_sync(0xffffffffu, P1, 0);
-        if (lane == 0) dn1 = b31;
-        if (lane == 31) {
-          up0 = b32;
-          up1 = 0.0;
-        }
-        P1 = fma(C[1], up1, fma(B[1], dn1, A[1] * P1));
-        acc1 = fma(c_inv_fact[k], P1, acc1);
-      } else {
-        if (lane == 31) up0 = 0.0;
-      }
-      P0 = fma(C[0], up0, fma(B[0], dn0, A[0] * P0));
-      acc0 = fma(c_inv_fact[k], P0, acc0);
+  double p0 = 0.0, p1 = 0.0, q0 = 0.0, q1 = 0.0, z0 = 0.0, z1 = 0.0;  // b_{k+1}, b_{k+2}, b_{k+3}
+  for (int k = n - 1; k >= 0; --k) {
+    const double tk = t[k];
+    double dn = __shfl_up_sync(0xffffffffu, TWO ? p1 : p0, 1);
+    const double up = __shfl_down_sync(0xffffffffu, p0, 1);
+    if (lane == 0) dn = tk;  // GEN: its coefficient is 0
+    double r0 = fma(B[0], dn, fma(A[0], p0, -q0)), r1 = 0.0;
+    if (TWO) {
+      r0 = fma(C[0], p1, r0);
+      r1 = fma(C[1], up, fma(B[1], p0, fma(A[1], p1, -q1)));
+    } else {
+      r0 = fma(C[0], up, r0);
     }
-    x[0] = acc0;
-    x[1] = acc1;
+    if (GEN) {
+      r0 = fma(tk, x[0], r0);
+      if (TWO) r1 = fma(tk, x[1], r1);
+    }
+    z0 = q0;
+    q0 = p0;
+    p0 = r0;
+    z1 = q1;
+    q1 = p1;
+    p1 = r1;
   }
+  // after k = 0: p = b_0, q = b_1, z = b_2
+  y[0] = 0.5 * (p0 - z0);
+  y[1] = TWO ? 0.5 * (p1 - z1) : 0.0;
 }
 
-static __device__ void small_expm_warp(const Ctl& c, int m, int p, double tau, double* yexp) {
+static __device__ __noinline__ void small_expm_warp(const Ctl& c, int m, int p, double tau, bool indef, double* yexp) {
   const int lane = threadIdx.x & 31;
-  const int M = m + p + 1;
-  // Gershgorin interval [L, U] of the augmented matrix (rows m.. have centre
-  // 0 and radius at most 1); FP32 suffices, it only picks the shift and the
-  // scaling.  exp(K) = e^mu exp(K - mu I) for any mu: mu is the interval's
-  // midpoint (floored at -300 so that neither factor overflows), which
-  // about halves the norm bound that sets the number of Taylor terms.
+  const int M = m + p + 1, na = p + 1;
+  // Gershgorin bounds of tau H_m (FP32, widened by 2^-20: they only place the
+  // interval)
   const float ft = (float)tau;
-  float L = -1.f, U = 1.f;
+  float L = -1.f, U = 0.f;
   for (int r = lane; r < m; r += 32) {
     const float cr = ft * (float)c.alpha[r];
-    const float rr = ft * ((r > 0 ? fabsf((float)c.low[r - 1]) : 0.f) + (r + 1 < m ? fabsf((float)c.up[r + 1]) : 0.f)) +
-                     (r == 0 ? 1.f : 0.f);
+    const float rr = ft * ((r > 0 ? fabsf((float)c.low[r - 1]) : 0.f) + (r + 1 < m ? fabsf((float)c.up[r + 1]) : 0.f));
     L = fminf(L, cr - rr);
     U = fmaxf(U, cr + rr);
   }
@@ -157,76 +204,108 @@ static __device__ void small_expm_warp(const Ctl& c, int m, int p, double tau, d
     L = fminf(L, __shfl_xor_sync(0xffffffffu, L, o));
     U = fmaxf(U, __shfl_xor_sync(0xffffffffu, U, o));
   }
-  const float mu = fmaxf(0.5f * (L + U), -300.f);
-  const float nb = fmaxf(U - mu, mu - L);
-  const int s = max(1, (int)ceilf(nb / TAYLOR_THETA));
-  const float th = nb / (float)s;
-  int deg = 1;
-  {
-    float term = th;
-    while (deg < 60 && term > 1e-18f) {
-      ++deg;
-      term *= __fdividef(th, (float)deg);
-    }
-  }
-  const double inv_s = 1.0 / (double)s;
-  const double dmu = (double)mu;
-  double A[2], B[2], C[2], x[2];
+  L *= 1.f + 0x1p-20f;
+  // the interval [L, n2 ln 2] in s steps of half-width a = 2^(i/2) each
+  int n2 = 0;
+  if (indef) n2 = (int)ceilf(fminf((U + 1.f) * 1.442696f, 1000.f));
+  float need = 0.5f * ((float)n2 * 0.6931472f - L);
+  const float top = indef ? 8.f : 512.f;
+  const int s = need > top ? (int)ceilf(fminf(need / top, 1e6f)) : 1;
+  need /= (float)s;
+  // smallest i with 2^(i/2) >= need
+  const int ex = (int)((__float_as_uint(fmaxf(need, 1.f)) >> 23) & 0xffu) - 127;
+  const float mant = __uint_as_float((__float_as_uint(fmaxf(need, 1.f)) & 0x7fffffu) | 0x3f800000u);
+  const int ia = min(2 * ex + (mant > 1.41421354f ? 2 : mant > 1.f ? 1 : 0), CHEB_TABLES - 1);
+  const double g = c_cheb_2a[ia];                       // 2 / a
+  double ts = g, shift = 2.0;                           // 2 X = ts K + shift
+  if (s > 1) ts = g / (double)s;
+  if (n2 > 0) shift = fma(-ts, (double)n2 * 0.6931471805599453, 2.0);
+  const double tt = ts * tau;
+  const bool two = M > 32;
+  double A[2], B[2], C[2], x[2], y[2];
+#pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const int r = lane + 32 * h;
-    if (r < m) {
-      A[h] = (tau * c.alpha[r] - dmu) * inv_s;
-      B[h] = r > 0 ? tau * c.low[r - 1] * inv_s : 0.0;
-      C[h] = r + 1 < m ? tau * c.up[r + 1] * inv_s : 0.0;
-    } else if (r < M) {
-      A[h] = -dmu * inv_s;
-      B[h] = 0.0;
-      C[h] = r < M - 1 ? inv_s : 0.0;
-    } else {
-      A[h] = B[h] = C[h] = 0.0;
+    const int j = two ? 2 * lane + h : lane + 32 * h;  // place in the chain
+    A[h] = B[h] = C[h] = x[h] = 0.0;
+    if (j < na) {
+      A[h] = shift;
+      B[h] = j > 0 ? ts : 0.0;
+    } else if (j < M) {
+      const int r = j - na;
+      A[h] = fma(tt, c.alpha[r], shift);
+      B[h] = r > 0 ? tt * c.low[r - 1] : ts;
+      C[h] = r + 1 < m ? tt * c.up[r + 1] : 0.0;
     }
-    x[h] = (r == M - 1) ? 1.0 : 0.0;
+    if (j == 0) x[h] = 1.0;
+    // the augmented rows' upper neighbours do not enter (C = 0)
   }
-  // row 0 has no lower neighbour: that slot carries its coupling to x_m
-  if (lane == 0) B[0] = inv_s;
-  if (M > 32) taylor_steps<true>(m, s, deg, A, B, C, x);
-  else taylor_steps<false>(m, s, deg, A, B, C, x);
-  const double emu = exp(dmu);
-  if (lane < m) yexp[lane] = x[0] * emu;
-  if (lane + 32 < m) yexp[lane + 32] = x[1] * emu;
+  const double* const t = c_cheb + c_cheb_at[ia];
+  const int n = c_cheb_at[ia + 1] - c_cheb_at[ia];
+  if (s == 1) {
+    if (lane == 0) B[0] = 1.0;
+    if (two) cheb_steps<true, false>(t, n, A, B, C, x, y);
+    else cheb_steps<false, false>(t, n, A, B, C, x, y);
+  } else {
+    for (int it = 0; it < s; ++it) {
+      if (two) cheb_steps<true, true>(t, n, A, B, C, x, y);
+      else cheb_steps<false, true>(t, n, A, B, C, x, y);
+      x[0] = y[0];
+      x[1] = y[1];
+    }
+  }
+  const double f = n2 > 0 ? scalbn(1.0, n2) : 1.0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int j = two ? 2 * lane + h : lane + 32 * h;
+    if (j >= na && j < M) yexp[j - na] = n2 > 0 ? y[h] * f : y[h];
+  }
   __syncwarp();
 }
 
 // Combination coefficients from yexp = phi_{p+1}(tau H_m) e_1 (one warp):
 // out_r = tau^p beta (phi_p(tau H_m) e_1)_r / |V_r|, with phi_p(X) e_1 =
 // X phi_{p+1}(X) e_1 + e_1 / p!  (p = 0 .. 3).
+__device__ __forceinline__ double tau_power(double tau, int p) {
+  return p == 0 ? 1.0 : p == 1 ? tau : p == 2 ? tau * tau : tau * tau * tau;
+}
 static __device__ void coef_row(const Ctl& c, int m, int p, double tau, const double* yexp, double* out) {
   const int lane = threadIdx.x & 31;
-  double taup = 1.0, invf = 1.0;
-  for (int i = 1; i <= p; ++i) {
-    taup *= tau;
-    invf /= (double)i;
-  }
+  const double tb = tau_power(tau, p) * c.beta;
+  const double invf = p <= 1 ? 1.0 : p == 2 ? 0.5 : 1.0 / 6.0;
   for (int r = lane; r < m; r += 32) {
     double hy = c.alpha[r] * yexp[r];
     if (r > 0) hy = fma(c.low[r - 1], yexp[r - 1], hy);
     if (r + 1 < m) hy = fma(c.up[r + 1], yexp[r + 1], hy);
     const double php = fma(tau, hy, r == 0 ? invf : 0.0);
-    out[r] = taup * c.beta * php * c.scale[r];
+    out[r] = tb * php * c.scale[r];
   }
   __syncwarp();
 }
+
+// x^(1/n), out of line (the controller's step factors)
+static __device__ __noinline__ double root_of(double x, int n) { return pow(x, 1.0 / n); }
 
 // After small_expm_warp: err and the combination coefficients (warp 0):
 // err = tau^{p+1} beta h_{m+1,m} |e_m^T phi_{p+1}(tau H_m) e_1|.
 static __device__ void finish_check(Ctl& c, int m, int p, double tau) {
   coef_row(c, m, p, tau, c.yexp, c.coef);
-  if ((threadIdx.x & 31) == 0) {
-    double taup = 1.0;
-    for (int i = 1; i <= p; ++i) taup *= tau;
-    c.err = taup * tau * c.beta * c.hn * fabs(c.yexp[m - 1]);
-  }
+  if ((threadIdx.x & 31) == 0) c.err = tau_power(tau, p) * tau * c.beta * c.hn * fabs(c.yexp[m - 1]);
   __syncwarp();
+}
+
+// The error check of the basis of c.m vectors at c.tau by warp 0 (every
+// thread of the block calls it and may read c.accepted after).  Out of line:
+// inlined at its call sites it costs the 768-thread kernel registers.
+static __device__ __noinline__ void check_basis(Ctl& c, int p, double tol, const int* negb) {
+  if (threadIdx.x < 32) {
+    small_expm_warp(c, c.m, p, c.tau, *negb != 0, c.yexp);
+    finish_check(c, c.m, p, c.tau);
+    if (threadIdx.x == 0) {
+      if (c.breakdown) c.err = 0.0;
+      c.accepted = c.err <= tol * c.tau * c.ynorm;
+    }
+  }
+  __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
@@ -909,12 +988,12 @@ __device__ __noinline__ void adj_lambda_outputs(const PhipmArgs<T>& a, const Spe
         for (int i = lane; i < m; i += 32) out[i] = c.beta * c.yexp[i] * c.scale[i];
         __syncwarp();
       } else if (r == 2) {
-        small_expm_warp(c, m, 1, 1.0, ye);
+        small_expm_warp(c, m, 1, 1.0, *S.negb != 0, ye);
         for (int i = lane; i < m; i += 32) out[i] = c.beta * ye[i] * c.scale[i];
         __syncwarp();
       } else {
         const double sq = a.tq[r - 3];
-        small_expm_warp(c, m, 0, sq, ye);
+        small_expm_warp(c, m, 0, sq, *S.negb != 0, ye);
         coef_row(c, m, 0, sq, ye, out);
       }
     }
@@ -965,7 +1044,7 @@ __device__ __noinline__ bool adj_y_outputs(const PhipmArgs<T>& a, const SpeciesD
   for (int r = wid; r < nr; r += nw) {
     double* out = rows + r * 64;
     if (m > 0) {
-      small_expm_warp(c, m, 2, s_shift[r], ye);
+      small_expm_warp(c, m, 2, s_shift[r], *S.negb != 0, ye);
       coef_row(c, m, 2, s_shift[r], ye, out);
     } else {
       for (int i = lane; i < 64; i += 32) out[i] = 0.0;
@@ -1084,6 +1163,61 @@ static __device__ __forceinline__ void quad_setup_etd2(const PhipmArgs<float>& a
   sums[0] = sy.value();
   sums[1] = s1.value();
   sums[2] = s2.value();
+}
+
+// The basis on the groups of 4 nodes from V_0, Z_0 and the state of a basis
+// of one vector: passes, sums and checks until the basis is accepted or
+// full.  Returns false if the kernel must stop.
+template <int N>
+__device__ __forceinline__ bool lanczos_quads(const PhipmArgs<float>& a, const SpeciesDev<float>& S, Ctl& c,
+                                           unsigned& bar, int& red, int P) {
+  const GridDev& g = a.g;
+  const long long gtid = dealt_tid();
+  const long long gthreads = (long long)gridDim.x * blockDim.x;
+  const float cfac = (float)a.cfac, bc = (float)S.beta_c, dint = quad_d_int<float, N>(S);
+  const double anorm = a.dt * (*S.gersh);
+  const int m_max = a.m_max;
+  const long long vs = g.size;
+  double* pb;
+  // Groups of 4 nodes: one pass per Krylov vector (quad_pass_1).
+  // Before pass j: alpha_{j-1}, beta_j and the scale s of V_{j-1}
+  // (1/|V_0| for V_0, 1 after); V_j = (u_{j-1} - alpha_{j-1} v_{j-1}) / beta_j
+  // with u_0 = A v_0 = s Z_0; u_j = A v_j - beta_j v_{j-1} -> Z[j & 1].
+  // After it: alpha_j = <u_j, V_j> / |V_j|^2, beta_{j+1}^2 =
+  // |u_j|^2 - <u_j, V_j>^2 / |V_j|^2; H is symmetric tridiagonal.
+  if (c.m == m_max || c.breakdown) check_basis(c, P, a.tol, S.negb);
+  for (int j = 1; j < m_max && !c.accepted; ++j) {
+    const double sp = c.scale[j - 1], bj = c.low[j - 1];
+    const float c1 = (float)(sp / bj), c2 = (float)(-c.alpha[j - 1] * sp / bj), c3 = (float)(-bj * sp);
+    const QuadSums qs = quad_pass_1<N>(S.Z[(j - 1) & 1], S.V + (long long)(j - 1) * vs, S.V + (long long)j * vs,
+                                       S.Z[j & 1], c1, c2, c3, S.kind, S.diagf, S.qidx, S.qk, c.nquad, g, cfac,
+                                       bc, dint, gtid, gthreads);
+    double v[3] = {qs.d1, qs.d2, qs.d3};
+    pb = part_buf(a.part, red);
+    block_partials<3>(v, pb);
+    if (!grid_barrier(a.st, bar, 13)) return false;
+    double tot[3];
+    grid_totals<3>(pb, tot);
+    if (threadIdx.x == 0) {
+      const double aj = tot[1] / tot[0];
+      const double bn = sqrt(fmax(tot[2] - tot[1] * aj, 0.0));
+      if (!isfinite(aj) || !isfinite(bn)) {
+        atomicOr(&a.st->err, ERRF_NONFINITE);
+        c.abort = 1;
+      }
+      c.alpha[j] = aj;
+      c.scale[j] = 1.0;
+      c.low[j] = bn;
+      c.up[j + 1] = bn;
+      c.hn = bn;
+      c.m = j + 1;
+      c.breakdown = bn < BREAKDOWN_REL * anorm;
+    }
+    __syncthreads();
+    if (c.abort) return false;
+    if (c.m % CHECK_EVERY == 0 || c.m == m_max || c.breakdown) check_basis(c, P, a.tol, S.negb);
+  }
+  return true;
 }
 
 template <typename T, int N, bool ADJ>
@@ -1295,58 +1429,9 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
       __syncthreads();
       if (c.abort) return false;
     }
-    // error check of the basis of c.m vectors (warp 0), then every thread reads c.accepted
-    const auto check = [&]() {
-      if (threadIdx.x < 32) {
-        small_expm_warp(c, c.m, P, c.tau, c.yexp);
-        finish_check(c, c.m, P, c.tau);
-        if (threadIdx.x == 0) {
-          if (c.breakdown) c.err = 0.0;
-          c.accepted = c.err <= a.tol * c.tau * c.ynorm;
-        }
-      }
-      __syncthreads();
-    };
     if (c.beta > 0.0 && quad) {
       if constexpr (sizeof(T) == 4) {
-        // Groups of 4 nodes: one pass per Krylov vector (quad_pass_1).
-        // Before pass j: alpha_{j-1}, beta_j and the scale s of V_{j-1}
-        // (1/|V_0| for V_0, 1 after); V_j = (u_{j-1} - alpha_{j-1} v_{j-1}) / beta_j
-        // with u_0 = A v_0 = s Z_0; u_j = A v_j - beta_j v_{j-1} -> Z[j & 1].
-        // After it: alpha_j = <u_j, V_j> / |V_j|^2, beta_{j+1}^2 =
-        // |u_j|^2 - <u_j, V_j>^2 / |V_j|^2; H is symmetric tridiagonal.
-        if (c.m == m_max || c.breakdown) check();
-        for (int j = 1; j < m_max && !c.accepted; ++j) {
-          const double sp = c.scale[j - 1], bj = c.low[j - 1];
-          const float c1 = (float)(sp / bj), c2 = (float)(-c.alpha[j - 1] * sp / bj), c3 = (float)(-bj * sp);
-          const QuadSums qs = quad_pass_1<N>(S.Z[(j - 1) & 1], S.V + (long long)(j - 1) * vs, S.V + (long long)j * vs,
-                                             S.Z[j & 1], c1, c2, c3, S.kind, S.diagf, S.qidx, S.qk, c.nquad, g, cfac,
-                                             bc, dint, gtid, gthreads);
-          double v[3] = {qs.d1, qs.d2, qs.d3};
-          pb = part_buf(a.part, red);
-          block_partials<3>(v, pb);
-          if (!grid_barrier(a.st, bar, 13)) return false;
-          double tot[3];
-          grid_totals<3>(pb, tot);
-          if (threadIdx.x == 0) {
-            const double aj = tot[1] / tot[0];
-            const double bn = sqrt(fmax(tot[2] - tot[1] * aj, 0.0));
-            if (!isfinite(aj) || !isfinite(bn)) {
-              atomicOr(&a.st->err, ERRF_NONFINITE);
-              c.abort = 1;
-            }
-            c.alpha[j] = aj;
-            c.scale[j] = 1.0;
-            c.low[j] = bn;
-            c.up[j + 1] = bn;
-            c.hn = bn;
-            c.m = j + 1;
-            c.breakdown = bn < BREAKDOWN_REL * anorm;
-          }
-          __syncthreads();
-          if (c.abort) return false;
-          if (c.m % CHECK_EVERY == 0 || c.m == m_max || c.breakdown) check();
-        }
+        if (!lanczos_quads<N>(a, S, c, bar, red, P)) return false;
       }
     }
     if (c.beta > 0.0) {
@@ -1467,7 +1552,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
           if (c.abort) return false;
         }
         if (c.m % CHECK_EVERY == 0 || c.m == m_max || c.breakdown) {
-          check();
+          check_basis(c, P, a.tol, S.negb);
           if (c.accepted) break;
         }
       }
@@ -1479,7 +1564,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
         for (;;) {
           if (threadIdx.x == 0) {
             const double tolabs = a.tol * c.tau * c.ynorm;
-            const double fac = fmax(0.2, 0.9 * pow(tolabs / c.err, 1.0 / (m + 1)));
+            const double fac = fmax(0.2, 0.9 * root_of(tolabs / c.err, m + 1));
             c.tau *= fac;
             c.last = 0;
             c.nrej += 1;
@@ -1490,12 +1575,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
           }
           __syncthreads();
           if (c.abort) return false;
-          if (threadIdx.x < 32) {
-            small_expm_warp(c, m, P, c.tau, c.yexp);
-            finish_check(c, m, P, c.tau);
-            if (threadIdx.x == 0) c.accepted = c.err <= a.tol * c.tau * c.ynorm;
-          }
-          __syncthreads();
+          check_basis(c, P, a.tol, S.negb);
           if (c.accepted) break;
         }
       }
@@ -1577,11 +1657,17 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
           st->rejections[sidx] += c.nrej;
           st->iters[sidx] += m;
         }
-        double grow;
-        if (c.err == 0.0) grow = 2.0;
-        else grow = fmin(2.0, 0.9 * pow(a.tol * c.tau * c.ynorm / c.err, 1.0 / (m + 1)));
-        c.t = c.last ? 1.0 : c.t + c.tau;
-        if (c.t < 1.0) c.tau = fmin(1.0 - c.t, c.tau * grow);
+        if (c.last) {
+          c.t = 1.0;
+        } else {
+          // (the last substep needs no next size: its pow is 100 dependent
+          // FP64 instructions)
+          double grow;
+          if (c.err == 0.0) grow = 2.0;
+          else grow = fmin(2.0, 0.9 * root_of(a.tol * c.tau * c.ynorm / c.err, m + 1));
+          c.t += c.tau;
+          if (c.t < 1.0) c.tau = fmin(1.0 - c.t, c.tau * grow);
+        }
         c.ynorm = fmax(fmax(sqrt(tot[0]), vscale), 1e-300);
         if (!isfinite(c.ynorm)) {
           atomicOr(&a.st->err, ERRF_NONFINITE);
@@ -1604,7 +1690,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
 // kept apart so that their code adds nothing to the other launches.  NT:
 // threads per CTA (one CTA per SM), which fixes the registers per thread.
 template <typename T, int N, bool ADJ, int NT>
-__global__ void __launch_bounds__(NT, 1) phipm_kernel(const PhipmArgs<T> a) {
+__global__ void __launch_bounds__(NT, 1) phipm_kernel(const __grid_constant__ PhipmArgs<T> a) {
   __shared__ Ctl c;
   unsigned bar = 0;
   int red = 0;
@@ -1885,7 +1971,7 @@ PhipmKernels phipm_kernels() {
   k.fn[2][1] = (void*)phipm_kernel<T, 4, true, NT>;
   k.nt = NT;
   k.adj_smem = adj_smem(NT);
-  k.load_consts = load_inv_fact;
+  k.load_consts = load_cheb;
   return k;
 }
 

@@ -176,6 +176,7 @@ extern "C" etd_status etd_phi_combination_noalloc(const etd_grid* grid, const do
   ma.diag = diag;
   ma.diagf = nullptr;
   ma.gersh = &dst->gersh[0];
+  ma.negb = &dst->negb[0];
   ma.st = dst;
   if (launch_init_domain(ca, ma, tiles, ncomp, st) != cudaSuccess) return ETD_ERR_CUDA;
 
@@ -196,6 +197,7 @@ extern "C" etd_status etd_phi_combination_noalloc(const etd_grid* grid, const do
   S.beta_field = nullptr;
   S.beta_c = beta;
   S.gersh = &dst->gersh[0];
+  S.negb = &dst->negb[0];
   S.u = y;
   S.V = V;
   S.Yg = Yg;
