@@ -77,6 +77,10 @@ struct LsArgs {
   int reinit;
   int mixed;  // FP32 WENO/Godunov arithmetic away from the interface
   WenoInt wi;  // constants of the integer WENO5 form
+  // constants of the grid, divided on the host: an FP64 division in every warp
+  // of the kernel takes an SM 2 us
+  double inv_h, inv_2h, band, ext_dtau, ext_dth, re_dtau, inv_h12;
+  float inv_hf;
 };
 
 LevelsetBufs levelset_carve(const GridDev& g, const std::function<char*(size_t)>& take) {
@@ -289,7 +293,7 @@ __device__ __forceinline__ double grad_int(const LsArgs& a, const StageLane<N>& 
     const double mx = godunov_mx_f64(f, positive, g.h);
     s = fma(mx, mx, s);
   }
-  return sqrt(s) * (1.0 / (12.0 * g.h));
+  return sqrt(s) * a.inv_h12;
 }
 
 // The same with the node's axes on N consecutive lanes (all lanes of the warp
@@ -331,7 +335,7 @@ __device__ __forceinline__ double grad_int_split(const LsArgs& a, const StageLan
       const double v = __shfl_sync(0xffffffffu, m, (base + d) & 31);
       s = fma(v, v, s);
     }
-    if (!all) gr = sqrt(s) * (1.0 / (12.0 * g.h));
+    if (!all) gr = sqrt(s) * a.inv_h12;
   }
   return gr;
 }
@@ -391,7 +395,7 @@ __device__ bool build_work_set(const LsArgs& a, LsCtx& c, bool with_valid, int s
   const GridDev& g = a.g;
   const BitGeo bg = bit_geo(g);
   uint32_t* const pl = a.b.bits;
-  const unsigned long long Gbits = (unsigned long long)__double_as_longlong(BAND * g.h);
+  const unsigned long long Gbits = (unsigned long long)__double_as_longlong(a.band);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   // row strides in words and row extents of the first N - 1 axes
   long long rsw[N > 1 ? N - 1 : 1];
@@ -881,8 +885,7 @@ __device__ bool ext_sweeps(const LsArgs& a, LsCtx& c, int n, long long cap, int 
 // clamped in integers as the FP64 path clamps the coordinate to the box.
 template <int N>
 __device__ double stefan_speed_f32(const GridDev& g, const double* __restrict__ u, const int* ix, const double* nv,
-                                   double ph, double mu) {
-  const float inv_h = (float)(1.0 / g.h);
+                                   double ph, double mu, float inv_h) {
   const float phf = (float)ph;
   const float hf = (float)g.h;
   float nf[N];
@@ -997,8 +1000,8 @@ struct StageDeal {
 template <int N, bool REINIT>
 __device__ bool rk3(const LsArgs& a, LsCtx& c, const StageDeal<N>& deal, StageLane<N>& e0, const double* rates,
                     int copies, double dt, bool clamp_last) {
-  const double G = BAND * a.g.h;
-  const float inv_h = (float)(1.0 / a.g.h);
+  const double G = a.band;
+  const float inv_h = a.inv_hf;
   for (int stage = 0; stage < 3; ++stage) {
     const auto run = [&](StageLane<N>& e, int chunk) {
       const bool positive = !REINIT || e.rate > 0.0;
@@ -1093,7 +1096,7 @@ __device__ bool reinitialise(const LsArgs& a, LsCtx& c) {
   }
   if (!grid_barrier(a.st, c.bar, 40)) return false;
   const int K = (int)ceil(12.0 * sqrt((double)N));
-  return rk3_steps<N, true>(a, c, a.b.S0, copies, K, 0.5 * h / sqrt((double)N));
+  return rk3_steps<N, true>(a, c, a.b.S0, copies, K, a.re_dtau);
 }
 
 template <int N>
@@ -1110,9 +1113,9 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
   }
   const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x, gth = (long long)gridDim.x * blockDim.x;
   const double h = g.h;
-  const double inv_h = 1.0 / h;
-  const double inv_2h = 0.5 * inv_h;
-  const double G = BAND * h;
+  const double inv_h = a.inv_h;
+  const double inv_2h = a.inv_2h;
+  const double G = a.band;
 
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     for (int i = 0; i < 8; ++i) a.b.info[i] = 0;
@@ -1273,8 +1276,8 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
   // is used in the rearranged form q' = c0 q + sum_d a_d q(up_d) + dtau s,
   // a_d = dtau |n_d| / h, c0 = 1 - sum_d a_d (equal up to rounding).
   const int K = (int)ceil(12.0 * sqrt((double)N));
-  const double dtau = h / (2.0 * sqrt((double)N));
-  const double dth = dtau * inv_h;
+  const double dtau = a.ext_dtau;
+  const double dth = a.ext_dth;
   {
     const double* const Q0[3] = {UNN[0], UN[0], U[0]};
     if (a.mixed) {
@@ -1299,7 +1302,7 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
       for (int d = 0; d < N; ++d) nv[d] = __ldcg(a.b.nrm + d * cap + i);
       double V;
       if (a.mixed) {
-        V = stefan_speed_f32<N>(g, a.u, ix, nv, ph, a.mu);
+        V = stefan_speed_f32<N>(g, a.u, ix, nv, ph, a.mu, a.inv_hf);
       } else {
         double xg[N];
 #pragma unroll
@@ -1352,9 +1355,16 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
   if (!grid_barrier(a.st, c.bar, 55)) return;
   // advection
   {
-    const double vmax = __ldcg(a.b.vmax);
-    double ns = ceil(a.dt * vmax * N / (0.5 * h));
-    int nsub = ns < 1.0 ? 1 : (int)fmin(ns, 1e6);
+    __shared__ double s_dts;
+    __shared__ int s_nsub;
+    if (threadIdx.x == 0) {
+      const double vmax = __ldcg(a.b.vmax);
+      const double ns = ceil(a.dt * vmax * N / (0.5 * h));
+      s_nsub = ns < 1.0 ? 1 : (int)fmin(ns, 1e6);
+      s_dts = a.dt / s_nsub;
+    }
+    __syncthreads();
+    const int nsub = s_nsub;
     if (nsub > 100000) {
       if (threadIdx.x == 0) atomicOr(&a.st->err, ERRF_NONFINITE);
       return;
@@ -1363,7 +1373,7 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
       *a.b.nsub = nsub;
       a.b.info[2] = nsub;
     }
-    if (!rk3_steps<N, false>(a, c, a.b.V, a.mixed ? COPY_F32 : COPY_INT, nsub, a.dt / nsub)) return;
+    if (!rk3_steps<N, false>(a, c, a.b.V, a.mixed ? COPY_F32 : COPY_INT, nsub, s_dts)) return;
   }
   if (a.reinit) reinitialise<N>(a, c);
 }
@@ -1375,6 +1385,19 @@ static int ls_blocks(int ndim) {
   void* fn = ndim == 2 ? (void*)levelset_kernel<2> : ndim == 3 ? (void*)levelset_kernel<3> : (void*)levelset_kernel<4>;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, LS_NT, 0) != cudaSuccess || per < 1) return 0;
   return min(sms, MAX_BLOCKS);
+}
+
+static void grid_consts(LsArgs& a, const GridDev& g) {
+  const double rn = sqrt((double)g.ndim);
+  a.wi = weno_int(g.h, WENO_EPS);
+  a.inv_h = 1.0 / g.h;
+  a.inv_2h = 0.5 * a.inv_h;
+  a.inv_h12 = 1.0 / (12.0 * g.h);
+  a.inv_hf = (float)a.inv_h;
+  a.band = BAND * g.h;
+  a.ext_dtau = g.h / (2.0 * rn);
+  a.ext_dth = a.ext_dtau * a.inv_h;
+  a.re_dtau = 0.5 * g.h / rn;
 }
 
 static cudaError_t launch(const LsArgs& a, cudaStream_t stream) {
@@ -1398,7 +1421,7 @@ cudaError_t launch_levelset_advance(const GridDev& g, const LevelsetBufs& b, Dev
                                     cudaStream_t stream) {
   LsArgs a;
   a.mixed = mixed ? 1 : 0;
-  a.wi = weno_int(g.h, WENO_EPS);
+  grid_consts(a, g);
   a.g = g;
   a.b = b;
   a.st = st;
@@ -1416,7 +1439,7 @@ cudaError_t launch_levelset_prepare(const GridDev& g, const LevelsetBufs& b, Dev
                                     bool mixed, cudaStream_t stream) {
   LsArgs a;
   a.mixed = mixed ? 1 : 0;
-  a.wi = weno_int(g.h, WENO_EPS);
+  grid_consts(a, g);
   a.g = g;
   a.b = b;
   a.st = st;
