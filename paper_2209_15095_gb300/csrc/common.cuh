@@ -5,11 +5,14 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "int64math.cuh"
+
 namespace etd {
 
 constexpr int MAXD = 4;
 constexpr int MAX_M = 61;           // largest Krylov basis (m + p + 1 <= 64)
 constexpr int MAX_BLOCKS = 1024;    // partial-sum slots per reduction quantity
+constexpr int MAX_SUM_BLOCKS = 256; // CTAs of a launch that uses GridSums
 
 // Unsigned division of n < 2^31 by a divisor d >= 1 fixed at set-up, on the
 // integer pipe: with s = ceil(log2 d) and m = floor(2^32 (2^s - d) / d) + 1,
@@ -218,6 +221,96 @@ __device__ __forceinline__ void grid_totals(const double* part, double (&out)[NQ
   __syncthreads();
 }
 
+// Sum of K values per lane over the warp, the same bits in every lane.  The
+// values are aligned to the largest exponent as 64-bit integers (rounded to
+// nearest at 2^-(57 - ceil(log2 K)) of the largest, below the rounding of an FP64
+// addition for K <= 8) and added exactly by three integer warp reductions: a
+// dependent FP64 addition takes about 70 cycles here and a tree of five with
+// their shuffles 500, this about 130.  Infinities, NaNs and sums near the ends of
+// the exponent range take FP64 additions.
+template <int K>
+__device__ __forceinline__ double warp_sum_int(const double (&v)[K]) {
+  constexpr int KB = K == 1 ? 0 : K == 2 ? 1 : K <= 4 ? 2 : 3;
+  static_assert(K <= 8, "too many values");
+  unsigned e = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k) e = max(e, ((unsigned)__double2hiint(v[k]) >> 20) & 0x7ffu);
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (e == 0u || e - 200u > 1600u) {
+    double x = 0.0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) x += v[k];
+    return e == 0u && !__any_sync(0xffffffffu, x != 0.0) ? 0.0 : warp_sum(x);
+  }
+  i64 f = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const u64 b = (u64)__double_as_longlong(v[k]);
+    const int ek = (int)((b >> 52) & 0x7ff);
+    const int r = (int)e - ek + 1;  // >= 1: one more bit for the rounding
+    u64 m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << (5 - KB);
+    m = ek == 0 || r > 62 ? 0ull : ((m >> (r - 1)) + 1ull) >> 1;
+    const i64 sg = (i64)b >> 63;
+    f += ((i64)m ^ sg) - sg;
+  }
+  // |f| < 2^57 in all: 22 + 22 + 14 bits
+  const int s0 = __reduce_add_sync(0xffffffffu, (int)(f & 0x3fffff));
+  const int s1 = __reduce_add_sync(0xffffffffu, (int)((f >> 22) & 0x3fffff));
+  const int s2 = __reduce_add_sync(0xffffffffu, (int)(f >> 44));
+  const i64 S = ((i64)s2 << 44) + ((i64)s1 << 22) + (i64)s0;
+  // units 2^(e - 1023 - 52 - 5 + KB + 1)
+  const double d = (double)S;
+  return S == 0 ? 0.0 : __longlong_as_double(__double_as_longlong(d) + ((i64)((int)e - 1023 - 56 + KB) << 52));
+}
+
+// Sums over the grid of NQ per-thread values, with a grid barrier: warp sums,
+// the CTA's sum by warp q for quantity q, the barrier, and all CTAs' sums by
+// warp q again, every CTA alike (the same bits everywhere).  Two sets of sums
+// alternate: between two that use the same set every CTA has passed a barrier
+// after reading it.  Returns false if the kernel must stop.
+struct GridSums {
+  double* part;  // 2 sets x 4 quantities x MAX_BLOCKS
+  int no;
+  __device__ __forceinline__ explicit GridSums(double* p) : part(p), no(0) {}
+  template <int NQ>
+  __device__ __forceinline__ bool sum(DevStatus* st, unsigned& bar, const double (&v)[NQ], double (&out)[NQ],
+                                      int site);
+};
+
+template <int NQ>
+__device__ __forceinline__ bool GridSums::sum(DevStatus* st, unsigned& bar, const double (&v)[NQ], double (&out)[NQ],
+                                              int site) {
+  __shared__ double s_w[NQ][32], s_out[NQ];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  double* const w = part + (size_t)(no & 1) * (4 * MAX_BLOCKS) + wid * MAX_BLOCKS;
+  ++no;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const double one[1] = {v[q]};
+    const double x = warp_sum_int<1>(one);
+    if (lane == 0) s_w[q][wid] = x;
+  }
+  __syncthreads();
+  if (wid < NQ) {
+    const double one[1] = {lane < nw ? s_w[wid][lane] : 0.0};
+    const double x = warp_sum_int<1>(one);
+    if (lane == 0) w[blockIdx.x] = x;
+  }
+  if (!grid_barrier(st, bar, site)) return false;
+  if (wid < NQ) {
+    constexpr int K = MAX_SUM_BLOCKS / 32;
+    double val[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) val[k] = 32 * k + lane < (int)gridDim.x ? __ldcg(w + 32 * k + lane) : 0.0;
+    const double t = warp_sum_int<K>(val);
+    if (lane == 0) s_out[wid] = t;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) out[q] = s_out[q];
+  return true;
+}
+
 // Exact widening to FP64.  For a float, normal values are widened on the
 // integer pipe (rebias the exponent, shift the mantissa): the hardware
 // conversion is an FP64-pipe instruction, which costs as much as an FMA.
@@ -270,7 +363,8 @@ struct Dot2f {
     s = t;
     c = __fadd_rn(c, __fadd_rn(e, pe));
   }
-  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+  // (a warp without points issues no FP64)
+  __device__ __forceinline__ double value() const { return s == 0.f && c == 0.f ? 0.0 : to_f64(s) + to_f64(c); }
 };
 
 template <typename T>

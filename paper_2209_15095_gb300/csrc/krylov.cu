@@ -46,7 +46,7 @@ cudaError_t launch_phipm(const PhipmArgs<T>& a, int nblocks, cudaStream_t stream
   const bool adj = a.mode == MODE_ADJ_LAMBDA || a.mode == MODE_ADJ_Y;
   if (a.g.ndim < 2 || a.g.ndim > 4) return cudaErrorInvalidValue;
   void* fn = v.k.fn[a.g.ndim - 2][adj ? 1 : 0];
-  if (nblocks > MAX_BLOCKS) return cudaErrorInvalidValue;
+  if (nblocks > MAX_SUM_BLOCKS) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(&a.st->barrier, 0, sizeof(unsigned), stream);
   if (e != cudaSuccess) return e;
   void* args[] = {(void*)&a};
@@ -76,7 +76,7 @@ int phipm_max_blocks(int ndim, bool fp32) {
       per = min(per, p);
     }
   }
-  return per * sms;
+  return min(per * sms, MAX_SUM_BLOCKS);
 }
 
 template cudaError_t launch_phipm<double>(const PhipmArgs<double>&, int, cudaStream_t, bool);

@@ -117,7 +117,10 @@ struct Ctl {
   float clo[MAX_M + 2];
   double yexp[64];
   // controller scalars
-  double t, tau, ynorm, beta, err, hn;
+  double t, tau, ynorm, vscale, beta, err, hn;
+  // coefficients of the next pass: of Z_{j-1}, V_{j-1}, V_{j-2} (FP32: as floats)
+  double cz, cv1, cv2;
+  float fz, fv1, fv2;
   int m, accepted, breakdown, last, abort, nrej;
   int trace0;  // trace entries of earlier launches of the step (block 0)
   int nquad, qoff;  // quad list: length, and this block's first entry
@@ -281,6 +284,9 @@ static __device__ void coef_row(const Ctl& c, int m, int p, double tau, const do
   }
   __syncwarp();
 }
+
+// whether x is finite, on its bits (an FP64 comparison costs as much as an FMA)
+__device__ __forceinline__ bool finite64(double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u; }
 
 // x^(1/n), out of line (the controller's step factors)
 static __device__ __noinline__ double root_of(double x, int n) { return pow(x, 1.0 / n); }
@@ -1168,9 +1174,18 @@ static __device__ __forceinline__ void quad_setup_etd2(const PhipmArgs<float>& a
 // The basis on the groups of 4 nodes from V_0, Z_0 and the state of a basis
 // of one vector: passes, sums and checks until the basis is accepted or
 // full.  Returns false if the kernel must stop.
+// The FP32 coefficients of pass j of the one-pass recurrence from the scale of
+// V_{j-1}, alpha_{j-1} and beta_j (one thread; every warp's own FP64 divisions
+// cost the SM 2 us per pass).
+__device__ __forceinline__ void quad_coefs(Ctl& c, double sp, double al, double bj) {
+  c.fz = (float)(sp / bj);
+  c.fv1 = (float)(-al * sp / bj);
+  c.fv2 = (float)(-bj * sp);
+}
+
 template <int N>
 __device__ __forceinline__ bool lanczos_quads(const PhipmArgs<float>& a, const SpeciesDev<float>& S, Ctl& c,
-                                           unsigned& bar, int& red, int P) {
+                                           unsigned& bar, GridSums& gs, int P) {
   const GridDev& g = a.g;
   const long long gtid = dealt_tid();
   const long long gthreads = (long long)gridDim.x * blockDim.x;
@@ -1178,7 +1193,6 @@ __device__ __forceinline__ bool lanczos_quads(const PhipmArgs<float>& a, const S
   const double anorm = a.dt * (*S.gersh);
   const int m_max = a.m_max;
   const long long vs = g.size;
-  double* pb;
   // Groups of 4 nodes: one pass per Krylov vector (quad_pass_1).
   // Before pass j: alpha_{j-1}, beta_j and the scale s of V_{j-1}
   // (1/|V_0| for V_0, 1 after); V_j = (u_{j-1} - alpha_{j-1} v_{j-1}) / beta_j
@@ -1187,21 +1201,17 @@ __device__ __forceinline__ bool lanczos_quads(const PhipmArgs<float>& a, const S
   // |u_j|^2 - <u_j, V_j>^2 / |V_j|^2; H is symmetric tridiagonal.
   if (c.m == m_max || c.breakdown) check_basis(c, P, a.tol, S.negb);
   for (int j = 1; j < m_max && !c.accepted; ++j) {
-    const double sp = c.scale[j - 1], bj = c.low[j - 1];
-    const float c1 = (float)(sp / bj), c2 = (float)(-c.alpha[j - 1] * sp / bj), c3 = (float)(-bj * sp);
+    const float c1 = c.fz, c2 = c.fv1, c3 = c.fv2;
     const QuadSums qs = quad_pass_1<N>(S.Z[(j - 1) & 1], S.V + (long long)(j - 1) * vs, S.V + (long long)j * vs,
                                        S.Z[j & 1], c1, c2, c3, S.kind, S.diagf, S.qidx, S.qk, c.nquad, g, cfac,
                                        bc, dint, gtid, gthreads);
     double v[3] = {qs.d1, qs.d2, qs.d3};
-    pb = part_buf(a.part, red);
-    block_partials<3>(v, pb);
-    if (!grid_barrier(a.st, bar, 13)) return false;
     double tot[3];
-    grid_totals<3>(pb, tot);
+    if (!gs.sum<3>(a.st, bar, v, tot, 13)) return false;
     if (threadIdx.x == 0) {
       const double aj = tot[1] / tot[0];
       const double bn = sqrt(fmax(tot[2] - tot[1] * aj, 0.0));
-      if (!isfinite(aj) || !isfinite(bn)) {
+      if (!finite64(aj) || !finite64(bn)) {
         atomicOr(&a.st->err, ERRF_NONFINITE);
         c.abort = 1;
       }
@@ -1212,6 +1222,7 @@ __device__ __forceinline__ bool lanczos_quads(const PhipmArgs<float>& a, const S
       c.hn = bn;
       c.m = j + 1;
       c.breakdown = bn < BREAKDOWN_REL * anorm;
+      quad_coefs(c, 1.0, aj, bn);
     }
     __syncthreads();
     if (c.abort) return false;
@@ -1222,7 +1233,7 @@ __device__ __forceinline__ bool lanczos_quads(const PhipmArgs<float>& a, const S
 
 template <typename T, int N, bool ADJ>
 __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int sidx, Ctl& c, unsigned& bar,
-                              int& red, double ynorm2, double vscale) {
+                              GridSums& gs, double ynorm2, double vnorm2) {
   const GridDev& g = a.g;
   const int ncomp = *S.ncomp;
   const long long gtid = dealt_tid();
@@ -1231,6 +1242,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
   const T bc = (T)S.beta_c;
   const float dint = quad_d_int<T, N>(S);  // the diagonal of the full groups (QK_FULL)
   const double anorm = a.dt * (*S.gersh);
+  const double brk = BREAKDOWN_REL * anorm;
   const int m_max = a.m_max;
   // highest phi index: 2 or 3 (any other value of a.p: 2); 0 for the basis
   // on lambda of the adjoint (V_0 = lambda, written by the set-up)
@@ -1251,11 +1263,14 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
   }
   // the statistics accumulate over the launches of one step (zeroed by the host)
   if (blockIdx.x == 0 && threadIdx.x == 0) c.trace0 = a.stats ? a.stats->trace_len[sidx] : 0;
-  double* pb = nullptr;
   if (threadIdx.x == 0) {
     c.t = 0.0;
     c.tau = 1.0;
-    c.ynorm = fmax(fmax(sqrt(ynorm2), vscale), 1e-300);
+    // (the roots by one thread: every warp's own take the SM 6 us)
+    double yn, r;
+    root_pair(vnorm2, c.vscale, r);
+    root_pair(ynorm2, yn, r);
+    c.ynorm = fmax(fmax(yn, c.vscale), 1e-300);
     c.abort = 0;
   }
   __syncthreads();
@@ -1357,13 +1372,13 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
     if (!grid_barrier(a.st, bar, 11)) return false;
     // P_0: Z_0 = A V_0, |V_0|^2, <Z_0, V_0> (and |Z_0|^2 on the 4-node groups)
     bool qp0 = false;
+    double tot[3] = {0.0, 0.0, 0.0};
     if constexpr (sizeof(T) == 4) {
       if (quad) {
         const QuadSums qs = quad_stencil<N, 0, true>(S.V, S.Z[0], nullptr, nullptr, nullptr, 0.f, 0.f, S.kind, S.diagf,
                                             S.qidx, S.qk, c.nquad, g, cfac, bc, dint, gtid, gthreads);
-        double v[3] = {qs.d1, qs.d2, qs.d3};
-        pb = part_buf(a.part, red);
-        block_partials<3>(v, pb);
+        const double v[3] = {qs.d1, qs.d2, qs.d3};
+        if (!gs.sum<3>(a.st, bar, v, tot, 12)) return false;
         qp0 = true;
       }
     }
@@ -1387,28 +1402,18 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
           d2.add(zz[u], vv[u]);
         }
       });
-      double v[2] = {d1.value(), d2.value()};
-      pb = part_buf(a.part, red);
-      block_partials<2>(v, pb);
+      const double v[3] = {d1.value(), d2.value(), 0.0};
+      if (!gs.sum<3>(a.st, bar, v, tot, 12)) return false;
     }
-    if (!grid_barrier(a.st, bar, 12)) return false;
     {
-      double tot[3] = {0.0, 0.0, 0.0};
-      if (quad) {
-        grid_totals<3>(pb, tot);
-      } else {
-        double t2[2];
-        grid_totals<2>(pb, t2);
-        tot[0] = t2[0];
-        tot[1] = t2[1];
-      }
       if (threadIdx.x == 0) {
-        c.beta = sqrt(tot[0]);
-        if (!isfinite(c.beta) || !isfinite(tot[1]) || !isfinite(tot[2])) {
+        double rbeta;
+        root_pair(tot[0], c.beta, rbeta);
+        if (!finite64(c.beta) || !finite64(tot[1]) || !finite64(tot[2])) {
           atomicOr(&a.st->err, ERRF_NONFINITE);
           c.abort = 1;
         }
-        const double s0 = c.beta > 0.0 ? 1.0 / c.beta : 0.0;
+        const double s0 = c.beta > 0.0 ? rbeta : 0.0;
         c.scale[0] = s0;
         c.alpha[0] = zfac * tot[1] * s0 * s0;
         c.up[0] = 0.0;
@@ -1424,6 +1429,15 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
           c.hn = b1;
           c.m = 1;
           c.breakdown = b1 < BREAKDOWN_REL * anorm;
+          quad_coefs(c, s0, c.alpha[0], b1);
+        }
+        c.cz = s0 * zfac;
+        c.cv1 = -c.alpha[0] * s0;
+        c.cv2 = 0.0;
+        if (sizeof(T) == 4 && !quad) {
+          c.fz = to_f32_rn(c.cz);
+          c.fv1 = to_f32_rn(c.cv1);
+          c.fv2 = 0.f;
         }
       }
       __syncthreads();
@@ -1431,7 +1445,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
     }
     if (c.beta > 0.0 && quad) {
       if constexpr (sizeof(T) == 4) {
-        if (!lanczos_quads<N>(a, S, c, bar, red, P)) return false;
+        if (!lanczos_quads<N>(a, S, c, bar, gs, P)) return false;
       }
     }
     if (c.beta > 0.0) {
@@ -1446,14 +1460,23 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
       // the same classical Gram-Schmidt coefficients as z = A v_j,
       // <z, v_j>, <z, v_{j-1}>, with the normalisation deferred.
       for (int j = 1; j <= m_max; ++j) {
-        const T ca = (T)(c.scale[j - 1] * zfac);              // coefficient of Z_{j-1}
-        const T cb = (T)(-c.alpha[j - 1] * c.scale[j - 1]);    // of V_{j-1}
-        const T cc = j >= 2 ? (T)(-c.up[j - 1] * c.scale[j - 2]) : T(0);  // of V_{j-2}
+        // coefficients of Z_{j-1}, V_{j-1}, V_{j-2}
+        T ca, cb, cc;
+        if constexpr (sizeof(T) == 8) {
+          ca = c.cz;
+          cb = c.cv1;
+          cc = c.cv2;
+        } else {
+          ca = c.fz;
+          cb = c.fv1;
+          cc = c.fv2;
+        }
         const T* Zp = S.Z[(j - 1) & 1];
         T* Zn = S.Z[j & 1];
         const T* V1 = S.V + (long long)(j - 1) * vs;
         const T* V2 = S.V + (long long)(j >= 2 ? j - 2 : 0) * vs;
         T* Vj = S.V + (long long)j * vs;
+        double sums[3];
         if (split) {
           // pass A_j: V_j = w_j at the own points only
           constexpr int U = SPLIT_U<T>;
@@ -1493,9 +1516,9 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
               d3.add(zv[u], v1v[u]);
             }
           });
-          double v[3] = {d1.value(), d2.value(), d3.value()};
-          pb = part_buf(a.part, red);
-          block_partials<3>(v, pb);
+          sums[0] = d1.value();
+          sums[1] = d2.value();
+          sums[2] = d3.value();
         } else {
           Acc<T> d1, d2, d3;
           for (long long k = gtid; k < ncomp; k += gthreads) {
@@ -1525,28 +1548,48 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
             d2.add(z, w);
             d3.add(z, v1);
           }
-          double v[3] = {d1.value(), d2.value(), d3.value()};
-          pb = part_buf(a.part, red);
-          block_partials<3>(v, pb);
+          sums[0] = d1.value();
+          sums[1] = d2.value();
+          sums[2] = d3.value();
         }
-        if (!grid_barrier(a.st, bar, 13)) return false;
+        double tot[3];
+        if (!gs.sum<3>(a.st, bar, sums, tot, 13)) return false;
         {
-          double tot[3];
-          grid_totals<3>(pb, tot);
-          if (threadIdx.x == 0) {
-            const double hn = sqrt(tot[0]);
-            if (!isfinite(hn) || !isfinite(tot[1]) || !isfinite(tot[2])) {
-              atomicOr(&a.st->err, ERRF_NONFINITE);
-              c.abort = 1;
+          // the Lanczos scalars and the next pass's coefficients by warp 0,
+          // products of the same form on lanes side by side: every FP64
+          // instruction of a warp takes 64 cycles here, whatever its lanes
+          if (threadIdx.x < 32) {
+            const int lane = threadIdx.x;
+            double hn, rhn;
+            root_pair(tot[0], hn, rhn);
+            const bool bd = __double_as_longlong(hn) < __double_as_longlong(brk);  // both non-negative
+            const double sj = bd ? 0.0 : rhn, sp = c.scale[j - 1];
+            // lane 0: h_jj = zfac tot1 sj^2; lane 1: h_{j-1,j} = zfac tot2 sj s_{j-1}
+            double h = (lane == 0 ? tot[1] : tot[2]) * sj * (lane == 0 ? sj : sp);
+            if (zb) h *= zfac;
+            // coefficients of Z_j (lane 2), V_j (lane 0), V_{j-1} (lane 1)
+            const double cf = lane == 2 ? sj * zfac : -h * (lane == 0 ? sj : sp);
+            if (lane == 0) {
+              if (!finite64(hn) || !finite64(tot[1]) || !finite64(tot[2])) {
+                atomicOr(&a.st->err, ERRF_NONFINITE);
+                c.abort = 1;
+              }
+              c.low[j - 1] = hn;
+              c.hn = hn;
+              c.m = j;
+              c.breakdown = bd;
+              c.scale[j] = sj;
+              c.alpha[j] = h;
+              c.cv1 = cf;
+              c.fv1 = to_f32_rn(cf);
+            } else if (lane == 1) {
+              c.up[j] = h;
+              c.cv2 = cf;
+              c.fv2 = to_f32_rn(cf);
+            } else if (lane == 2) {
+              c.cz = cf;
+              c.fz = to_f32_rn(cf);
             }
-            c.low[j - 1] = hn;
-            c.hn = hn;
-            c.m = j;
-            c.breakdown = hn < BREAKDOWN_REL * anorm;
-            const double sj = c.breakdown ? 0.0 : 1.0 / hn;
-            c.scale[j] = sj;
-            c.alpha[j] = zfac * tot[1] * sj * sj;
-            c.up[j] = zfac * tot[2] * sj * c.scale[j - 1];
           }
           __syncthreads();
           if (c.abort) return false;
@@ -1637,14 +1680,10 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
         S.Yg[p] = (T)y;
         yn.add(y, y);
       }
-      double v[1] = {yn.value()};
-      pb = part_buf(a.part, red);
-      block_partials<1>(v, pb);
+      const double v[3] = {yn.value(), 0.0, 0.0};
+      if (!gs.sum<3>(a.st, bar, v, tot, 14)) return false;
     }
-    if (!grid_barrier(a.st, bar, 14)) return false;
     {
-      double tot[1];
-      grid_totals<1>(pb, tot);
       if (threadIdx.x == 0) {
         const int m = c.m;
         if (blockIdx.x == 0 && a.stats) {
@@ -1668,8 +1707,10 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
           c.t += c.tau;
           if (c.t < 1.0) c.tau = fmin(1.0 - c.t, c.tau * grow);
         }
-        c.ynorm = fmax(fmax(sqrt(tot[0]), vscale), 1e-300);
-        if (!isfinite(c.ynorm)) {
+        double yn, r;
+        root_pair(tot[0], yn, r);
+        c.ynorm = fmax(fmax(yn, c.vscale), 1e-300);
+        if (!finite64(c.ynorm)) {
           atomicOr(&a.st->err, ERRF_NONFINITE);
           c.abort = 1;
         }
@@ -1694,7 +1735,7 @@ __global__ void __launch_bounds__(NT, 1) phipm_kernel(const __grid_constant__ Ph
   __shared__ Ctl c;
   unsigned bar = 0;
   int red = 0;
-  double* pb = nullptr;
+  GridSums gs(a.part);
   const GridDev& g = a.g;
   const long long gtid = dealt_tid();
   const long long gthreads = (long long)gridDim.x * blockDim.x;
@@ -1850,31 +1891,25 @@ __global__ void __launch_bounds__(NT, 1) phipm_kernel(const __grid_constant__ Ph
         }
       });
     }
-    sums[s][0] = acc.value() + at.value();
-    sums[s][1] = acc1.value() + at1.value();
-    sums[s][2] = acc2.value() + at2.value();
-    sums[s][3] = acc3.value() + at3.value();
+    if (a.mode == MODE_STAGE) {
+      sums[s][0] = acc.value();
+      sums[s][1] = acc1.value();
+      sums[s][2] = acc2.value();
+      sums[s][3] = acc3.value();
+    } else {
+      sums[s][0] = at.value();
+      sums[s][1] = at1.value();
+      sums[s][2] = at2.value();
+      sums[s][3] = at3.value();
+    }
   }
-  // |y(0)|^2, |v_1|^2, |v_2|^2, |v_3|^2 per species (one grid barrier each;
-  // two block sums of two quantities into the halves of one partial buffer)
+  // |y(0)|^2, |v_1|^2, |v_2|^2, |v_3|^2 per species (one grid barrier each)
   double tot[2][4];
+  for (int s = 0; s < a.nspecies; ++s)
+    if (!gs.sum<4>(a.st, bar, sums[s], tot[s], 1)) return;
   for (int s = 0; s < a.nspecies; ++s) {
-    double v01[2] = {sums[s][0], sums[s][1]}, v23[2] = {sums[s][2], sums[s][3]};
-    pb = part_buf(a.part, red);
-    block_partials<2>(v01, pb);
-    block_partials<2>(v23, pb + 2 * MAX_BLOCKS);
-    if (!grid_barrier(a.st, bar, 1)) return;
-    double t01[2], t23[2];
-    grid_totals<2>(pb, t01);
-    grid_totals<2>(pb + 2 * MAX_BLOCKS, t23);
-    tot[s][0] = t01[0];
-    tot[s][1] = t01[1];
-    tot[s][2] = t23[0];
-    tot[s][3] = t23[1];
-  }
-  for (int s = 0; s < a.nspecies; ++s) {
-    const double vscale = fmax(fmax(sqrt(tot[s][1]), sqrt(tot[s][2])), sqrt(tot[s][3]));
-    if (!phipm_species<T, N, ADJ>(a, a.sp[s], s, c, bar, red, tot[s][0], vscale)) return;
+    const double vnorm2 = fmax(fmax(tot[s][1], tot[s][2]), tot[s][3]);
+    if (!phipm_species<T, N, ADJ>(a, a.sp[s], s, c, bar, gs, tot[s][0], vnorm2)) return;
   }
   if (!grid_barrier(a.st, bar, 2)) return;
   // the adjoint modes' outputs are written by the species loop
