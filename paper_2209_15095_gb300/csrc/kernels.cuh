@@ -184,6 +184,7 @@ struct PoissonArgs {
   const double* f;       // full grid: right-hand side
   double* u;             // full grid: initial guess in, solution out (computational points)
   double tol;            // relative residual |r| / |b - f|
+  double cfac;           // 1 / h^2 (set by the launch)
   int max_iter;
   double* part;
   DevStatus* st;
