@@ -933,7 +933,10 @@ etd_status etd_read_domain(etd_ctx* c, int species, int* ncomp, int* nclamp, dou
   if (e != cudaSuccess) return cuda_fail(c, e, "read ncomp");
   if (ncomp) *ncomp = nc;
   if (nclamp) cudaMemcpy(nclamp, &c->st->nclamp, sizeof(int), cudaMemcpyDeviceToHost);
-  if (gersh) cudaMemcpy(gersh, &c->st->gersh[species], sizeof(double), cudaMemcpyDeviceToHost);
+  if (gersh) {
+    cudaMemcpy(gersh, &c->st->gersh[species], sizeof(double), cudaMemcpyDeviceToHost);
+    *gersh /= c->g.h * c->g.h;
+  }
   if (kind) cudaMemcpy(kind, b.kind, (size_t)c->g.size, cudaMemcpyDeviceToHost);
   const int n = nc < cap ? nc : cap;
   if (idx && n > 0) cudaMemcpy(idx, b.idx, sizeof(int) * n, cudaMemcpyDeviceToHost);

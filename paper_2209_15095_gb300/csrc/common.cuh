@@ -73,7 +73,7 @@ struct DevStatus {
   int nclamp;           // ghost weights clamped to [0, 1]
   int timeout_site;
   int pad;
-  double gersh[2];      // Gershgorin bound of C per species (max row sum of |C|)
+  double gersh[2];      // Gershgorin bound of h^2 C per species (max row sum of |h^2 C|)
   unsigned int barrier; // grid-barrier arrival counter (reset before each cooperative launch)
   unsigned int pad2;
   int negb[2];          // per species: the beta field has a negative value

@@ -150,48 +150,65 @@ __device__ __forceinline__ void atomic_max_pos(double* a, double v) {
   atomicMax((unsigned long long*)a, (unsigned long long)__double_as_longlong(v));
 }
 
-// Class of a node from phi: inside (phi < 0) with all 2N axis neighbours
-// inside and not on the box boundary is computational, inside otherwise a
-// ghost; near flags inside-or-not nodes within 3 of the boundary.  Loading
-// (node_load) is split from deciding (node_class) so that a warp issues the
-// loads of several words before it waits on any of them; neighbour indices
-// are clamped into the box (an edge node is a ghost or outside whatever they
-// hold).  Grids hold fewer than 2^31 nodes: 32-bit index arithmetic.
-template <int N>
-struct NodeLoad {
-  double v, w[2 * N];
-  bool edge, near;
-};
-
-template <int N>
-__device__ __forceinline__ void node_load(const GridDev& g, const double* __restrict__ phi, long long p,
-                                          NodeLoad<N>& L) {
-  unsigned rem = (unsigned)p;
-  L.edge = false;
-  L.near = false;
-  long long nb[2 * N];
-#pragma unroll
-  for (int d = 0; d < N; ++d) {
-    const unsigned st = (unsigned)g.stride[d];
-    const int i = (int)g.sdiv[d].div(rem);
-    rem -= (unsigned)i * st;
-    if (i == 0 || i == g.n[d] - 1) L.edge = true;
-    if (i < 3 || i > g.n[d] - 4) L.near = true;
-    nb[2 * d] = i > 0 ? p - g.stride[d] : p;
-    nb[2 * d + 1] = i < g.n[d] - 1 ? p + g.stride[d] : p;
+// The bit plane sbits (bit b of word w: node 32 w + b) moved by o nodes: bit b of
+// the result is that of node 32 w + b + o (FWD) or 32 w + b - o, o > 0, and 0
+// where that lies outside the plane of nw words.
+template <bool FWD>
+__device__ __forceinline__ unsigned shifted_word(const uint32_t* __restrict__ sbits, long long w, long long nw,
+                                                 long long o) {
+  const long long q = o >> 5;
+  const int s = (int)(o & 31);
+  if (FWD) {
+    const unsigned lo = w + q < nw ? __ldcg(sbits + w + q) : 0u;
+    if (s == 0) return lo;
+    return __funnelshift_r(lo, w + q + 1 < nw ? __ldcg(sbits + w + q + 1) : 0u, s);
   }
-  L.v = phi[p];
-#pragma unroll
-  for (int j = 0; j < 2 * N; ++j) L.w[j] = phi[nb[j]];
+  const unsigned hi = w - q >= 0 ? __ldcg(sbits + w - q) : 0u;
+  if (s == 0) return hi;
+  return __funnelshift_l(w - q - 1 >= 0 ? __ldcg(sbits + w - q - 1) : 0u, hi, s);
 }
 
+// Which of the nodes 32 w .. 32 w + 31 lie on the box boundary (edge) and
+// within 3 nodes of it (near), row by row (a word spans up to two rows of 32
+// nodes or more, up to five of 8).
 template <int N>
-__device__ __forceinline__ uint8_t node_class(const NodeLoad<N>& L) {
-  if (!negative(L.v)) return K_OUT;
-  bool all = !L.edge;
+__device__ __forceinline__ void edge_masks(const GridDev& g, long long w, unsigned& edge, unsigned& near) {
+  const int nx = g.n[N - 1];
+  edge = near = 0u;
+  int b = 0;
+  while (b < 32 && 32 * w + b < g.size) {
+    int ix[N];
+    unsigned rem = (unsigned)(32 * w + b);
 #pragma unroll
-  for (int j = 0; j < 2 * N; ++j) all = all && negative(L.w[j]);
-  return all ? K_COMP : K_GHOST;
+    for (int d = 0; d < N; ++d) {
+      ix[d] = (int)g.sdiv[d].div(rem);
+      rem -= (unsigned)ix[d] * (unsigned)g.stride[d];
+    }
+    const int x0 = ix[N - 1], len = min(32 - b, nx - x0);
+    const unsigned seg = (len == 32 ? 0xffffffffu : (1u << len) - 1u) << b;
+    bool on = false, by = false;
+#pragma unroll
+    for (int d = 0; d < N - 1; ++d) {
+      on = on || ix[d] == 0 || ix[d] == g.n[d] - 1;
+      by = by || ix[d] < 3 || ix[d] > g.n[d] - 4;
+    }
+    if (on) edge |= seg;
+    if (by) near |= seg;
+    // the row's first and last nodes that fall into the segment
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int l = k - x0, r = nx - 1 - k - x0;
+      if (l >= 0 && l < len) {
+        near |= 1u << (b + l);
+        if (k == 0) edge |= 1u << (b + l);
+      }
+      if (r >= 0 && r < len) {
+        near |= 1u << (b + r);
+        if (k == 0) edge |= 1u << (b + r);
+      }
+    }
+    b += len;
+  }
 }
 
 // Phase 3: per computational row, D_p and the Gershgorin row sum.  One
@@ -260,9 +277,11 @@ __device__ void metadata_phase(const MetaArgs& a, int ncomp) {
         const long long r = q + s;
         double wv;
         if (!negative(a.phi[r])) {
-          const double theta = a.phi[q] / (a.phi[q] - a.phi[r]);
-          wv = theta / (1.0 + theta);
+          // theta / (1 + theta) with theta = phi_q / (phi_q - phi_r), in one division
+          const double phq = a.phi[q], den = phq - a.phi[r];
+          wv = phq / (den + phq);
           if (a.bco) {
+            const double theta = phq / den;
             // case 2: the crossing at x_q + s theta h e_d, weight 1 / (1 + theta)
             bc[0] = bf * (1.0 / (1.0 + theta)) / h2;
 #pragma unroll
@@ -323,12 +342,12 @@ __device__ void metadata_phase(const MetaArgs& a, int ncomp) {
     if (act && f == 0) {
       a.diag[k] = D;
       if (a.diagf) a.diagf[k] = (float)D;
-      if (!interior) gmax = fmax(gmax, (D + off) / h2);
+      if (!interior) gmax = fmax(gmax, D + off);
       seen_interior = seen_interior || interior;
     }
   }
   // the interior rows' Gershgorin sum, once for all of those this thread wrote
-  if (seen_interior) gmax = fmax(gmax, (D_int + D_int) / h2);
+  if (seen_interior) gmax = fmax(gmax, D_int + D_int);
   for (int o = 16; o > 0; o >>= 1) {
     gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
     nclamp += __shfl_xor_sync(0xffffffffu, nclamp, o);
@@ -367,131 +386,78 @@ __global__ void __launch_bounds__(INIT_NT, 1) init_domain_kernel(const ClassifyA
   __shared__ int s_w[INIT_NT / 32];
   __shared__ int s_off, s_tot;
   int cnt = 0;
-  constexpr int UW = 4;  // words per warp and iteration: their loads overlap
-  const int nx = g.n[N - 1];
-  if ((nx & 31) == 0) {
-    // Rows are whole 32-node words: classify a word at a time from a sign
-    // plane (bit set where phi < 0).  A node is computational when it and its
-    // 2N neighbours are inside and it is not on the box edge; the x
-    // neighbours are the word shifted by one bit (with the end bits of the
-    // adjacent words), the others the words one stride away.
-    uint32_t* const sbits = cbits + nw;
-    constexpr int US = 16;  // words per warp and iteration of the sign plane
-    for (long long w0 = wlo + (long long)wid * US; w0 < whi; w0 += (long long)nwarp * US) {
-      double v[US];
+  // Classification 32 nodes at a time from a sign plane (bit set where phi <
+  // 0): a node is computational when it and its 2N neighbours are inside and it
+  // is not on the box boundary; the neighbours' bits are the plane moved by a
+  // stride.  A node that is inside within 3 nodes of the boundary is an error,
+  // so a moved word's bits from the next row reach no node that counts, but
+  // the boundary nodes themselves, which are masked off.
+  uint32_t* const sbits = cbits + nw;
+  constexpr int US = 16;  // words per warp and iteration of the sign plane
+  for (long long w0 = wlo + (long long)wid * US; w0 < whi; w0 += (long long)nwarp * US) {
+    double v[US];
 #pragma unroll
-      for (int u = 0; u < US; ++u) v[u] = w0 + u < whi ? ca.phi[32 * (w0 + u) + lane] : 1.0;
-#pragma unroll
-      for (int u = 0; u < US; ++u) {
-        const unsigned b = __ballot_sync(0xffffffffu, negative(v[u]));
-        if (lane == 0 && w0 + u < whi) sbits[w0 + u] = b;
-      }
+    for (int u = 0; u < US; ++u) {
+      const long long p = 32 * (w0 + u) + lane;
+      v[u] = w0 + u < whi && p < g.size ? ca.phi[p] : 1.0;
     }
-    if (!grid_barrier(ca.st, bar, 62)) return;
-    // a thread per word: its 32 kinds are written as two 16-byte stores
-    for (long long w = wlo + threadIdx.x; w < whi; w += blockDim.x) {
-      // axis indices of the word's first node
-      int ix[N];
-      unsigned rem = (unsigned)(32 * w);
 #pragma unroll
-      for (int d = 0; d < N; ++d) {
-        ix[d] = (int)g.sdiv[d].div(rem);
-        rem -= (unsigned)ix[d] * (unsigned)g.stride[d];
-      }
-      const int x0 = ix[N - 1];
-      const unsigned s0 = __ldcg(sbits + w);
-      const unsigned sl = x0 > 0 ? __ldcg(sbits + w - 1) : 0u;
-      const unsigned sr = x0 + 32 < nx ? __ldcg(sbits + w + 1) : 0u;
-      unsigned all = s0 & ((s0 << 1) | (sl >> 31)) & ((s0 >> 1) | (sr << 31));
-      unsigned nearm = 0u;  // nodes within 3 nodes of the box edge
-#pragma unroll
-      for (int d = 0; d < N - 1; ++d) {
-        const long long ws = g.stride[d] >> 5;
-        all &= ix[d] > 0 ? __ldcg(sbits + w - ws) : 0u;
-        all &= ix[d] < g.n[d] - 1 ? __ldcg(sbits + w + ws) : 0u;
-        if (ix[d] < 3 || ix[d] > g.n[d] - 4) nearm = 0xffffffffu;
-      }
-      if (x0 == 0) {
-        all &= ~1u;
-        nearm |= 0x7u;
-      }
-      if (x0 + 32 == nx) {
-        all &= 0x7fffffffu;
-        nearm |= 0xe0000000u;
-      }
-      if (s0 & nearm) atomicOr(&ca.st->err, ERRF_DOMAIN);
-      // kind byte = inside bit + computational bit (K_OUT 0, K_GHOST 1,
-      // K_COMP 2); a nibble spreads to one bit per byte by a multiply
-      uint4* const kp = reinterpret_cast<uint4*>(ca.kind + 32 * w);
-      const uint4 o0 = kp[0], o1 = kp[1];
-      const unsigned ow[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
-      unsigned kw[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        kw[q] = ((((s0 >> (4 * q)) & 15u) * 0x204081u) & 0x01010101u) +
-                ((((all >> (4 * q)) & 15u) * 0x204081u) & 0x01010101u);
-        // nodes that stop being computational: zero their vector entries
-        unsigned z = (ow[q] >> 1) & ~(kw[q] >> 1) & 0x01010101u;
-        while (z) {
-          const long long p = 32 * w + 4 * q + ((__ffs(z) - 1) >> 3);
-          z &= z - 1u;
-          for (int s = 0; s < ca.nzero; ++s) {
-            if (ca.zero_f64[s]) ca.zero_f64[s][p] = 0.0;
-            if (ca.zero_f32[s]) ca.zero_f32[s][p] = 0.0f;
-          }
-          for (int j = 0; j < ca.nbasis; ++j) {
-            if (ca.basis_f64) ca.basis_f64[(long long)j * g.size + p] = 0.0;
-            if (ca.basis_f32) ca.basis_f32[(long long)j * g.size + p] = 0.0f;
-          }
-        }
-      }
-      kp[0] = make_uint4(kw[0], kw[1], kw[2], kw[3]);
-      kp[1] = make_uint4(kw[4], kw[5], kw[6], kw[7]);
-      cbits[w] = all;
-      cnt += __popc(all);
-    }
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-  } else {
-    for (long long w0 = wlo + (long long)wid * UW; w0 < whi; w0 += (long long)nwarp * UW) {
-      NodeLoad<N> L[UW];
-      uint8_t old[UW];
-      bool val[UW];
-  #pragma unroll
-      for (int u = 0; u < UW; ++u) {
-        const long long p = 32 * (w0 + u) + lane;
-        val[u] = w0 + u < whi && p < g.size;
-        old[u] = K_OUT;
-        if (val[u]) {
-          node_load<N>(g, ca.phi, p, L[u]);
-          old[u] = ca.kind[p] & 3;
-        }
-      }
-  #pragma unroll
-      for (int u = 0; u < UW; ++u) {
-        const long long p = 32 * (w0 + u) + lane;
-        const uint8_t k = val[u] ? node_class<N>(L[u]) : K_OUT;
-        if (val[u]) {
-          if (k != K_OUT && L[u].near) atomicOr(&ca.st->err, ERRF_DOMAIN);
-          if (old[u] == K_COMP && k != K_COMP) {
-            for (int s = 0; s < ca.nzero; ++s) {
-              if (ca.zero_f64[s]) ca.zero_f64[s][p] = 0.0;
-              if (ca.zero_f32[s]) ca.zero_f32[s][p] = 0.0f;
-            }
-            for (int j = 0; j < ca.nbasis; ++j) {
-              if (ca.basis_f64) ca.basis_f64[(long long)j * g.size + p] = 0.0;
-              if (ca.basis_f32) ca.basis_f32[(long long)j * g.size + p] = 0.0f;
-            }
-          }
-          ca.kind[p] = k;
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, val[u] && k == K_COMP);
-        if (lane == 0 && w0 + u < whi) {
-          cbits[w0 + u] = bal;
-          cnt += __popc(bal);
-        }
-      }
+    for (int u = 0; u < US; ++u) {
+      const unsigned b = __ballot_sync(0xffffffffu, negative(v[u]));
+      if (lane == 0 && w0 + u < whi) sbits[w0 + u] = b;
     }
   }
+  if (!grid_barrier(ca.st, bar, 62)) return;
+  // a thread per word: its 32 kinds are written as two 16-byte stores (the
+  // arrays are padded to whole words)
+  for (long long w = wlo + threadIdx.x; w < whi; w += blockDim.x) {
+    const unsigned s0 = __ldcg(sbits + w);
+    unsigned all = s0;
+    if (s0) {
+#pragma unroll
+      for (int d = 0; d < N; ++d)
+        all &= shifted_word<true>(sbits, w, nw, g.stride[d]) & shifted_word<false>(sbits, w, nw, g.stride[d]);
+      unsigned edge, near;
+      edge_masks<N>(g, w, edge, near);
+      all &= ~edge;
+      if (s0 & near) atomicOr(&ca.st->err, ERRF_DOMAIN);
+    }
+    // kind byte = inside bit + computational bit (K_OUT 0, K_GHOST 1,
+    // K_COMP 2); a nibble spreads to one bit per byte by a multiply
+    uint4* const kp = reinterpret_cast<uint4*>(ca.kind + 32 * w);
+    const uint4 o0 = kp[0], o1 = kp[1];
+    const unsigned ow[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
+    unsigned kw[8];
+    unsigned changed = 0u;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      kw[q] = ((((s0 >> (4 * q)) & 15u) * 0x204081u) & 0x01010101u) +
+              ((((all >> (4 * q)) & 15u) * 0x204081u) & 0x01010101u);
+      changed |= kw[q] ^ ow[q];
+      // nodes that stop being computational: zero their vector entries
+      unsigned z = (ow[q] >> 1) & ~(kw[q] >> 1) & 0x01010101u;
+      while (z) {
+        const long long p = 32 * w + 4 * q + ((__ffs(z) - 1) >> 3);
+        z &= z - 1u;
+        if (p >= g.size) break;
+        for (int s = 0; s < ca.nzero; ++s) {
+          if (ca.zero_f64[s]) ca.zero_f64[s][p] = 0.0;
+          if (ca.zero_f32[s]) ca.zero_f32[s][p] = 0.0f;
+        }
+        for (int j = 0; j < ca.nbasis; ++j) {
+          if (ca.basis_f64) ca.basis_f64[(long long)j * g.size + p] = 0.0;
+          if (ca.basis_f32) ca.basis_f32[(long long)j * g.size + p] = 0.0f;
+        }
+      }
+    }
+    if (changed) {
+      kp[0] = make_uint4(kw[0], kw[1], kw[2], kw[3]);
+      kp[1] = make_uint4(kw[4], kw[5], kw[6], kw[7]);
+    }
+    cbits[w] = all;
+    cnt += __popc(all);
+  }
+  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
   if (lane == 0) s_w[wid] = cnt;
   __syncthreads();
   if (threadIdx.x == 0) {

@@ -1190,7 +1190,7 @@ __device__ __forceinline__ bool lanczos_quads(const PhipmArgs<float>& a, const S
   const long long gtid = dealt_tid();
   const long long gthreads = (long long)gridDim.x * blockDim.x;
   const float cfac = (float)a.cfac, bc = (float)S.beta_c, dint = quad_d_int<float, N>(S);
-  const double anorm = a.dt * (*S.gersh);
+  const double anorm = a.cfac * (*S.gersh);
   const int m_max = a.m_max;
   const long long vs = g.size;
   // Groups of 4 nodes: one pass per Krylov vector (quad_pass_1).
@@ -1241,7 +1241,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
   const T cfac = (T)a.cfac;
   const T bc = (T)S.beta_c;
   const float dint = quad_d_int<T, N>(S);  // the diagonal of the full groups (QK_FULL)
-  const double anorm = a.dt * (*S.gersh);
+  const double anorm = a.cfac * (*S.gersh);
   const double brk = BREAKDOWN_REL * anorm;
   const int m_max = a.m_max;
   // highest phi index: 2 or 3 (any other value of a.p: 2); 0 for the basis
