@@ -400,11 +400,7 @@ etd_status run_phipm(etd_ctx* c, int mode, double dt, double* const* u, int spec
   a.part = c->part;
   a.st = c->st;
   a.stats = c->stats;
-  cudaError_t e = cudaSuccess;
-  if (!keep_stats) {
-    e = cudaMemsetAsync(c->stats, 0, sizeof(StatsDev), c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "stats reset");
-  }
+  a.keep_stats = keep_stats ? 1 : 0;
   // the 768-thread FP32 kernel when a species of this launch takes the
   // 4-node groups (its latest known point count; only the speed depends on it)
   bool wide = false;
@@ -419,7 +415,7 @@ etd_status run_phipm(etd_ctx* c, int mode, double dt, double* const* u, int spec
                       c->g.n[c->g.ndim - 1] % 4 == 0);
     }
   }
-  e = launch_phipm<T>(a, c->nblocks, c->stream, wide);
+  cudaError_t e = launch_phipm<T>(a, c->nblocks, c->stream, wide);
   if (e != cudaSuccess) return cuda_fail(c, e, "phipm launch");
   c->last_nspecies = a.nspecies;
   c->last_species0 = all ? 0 : species;
@@ -580,9 +576,7 @@ etd_status etd_init_domain(etd_ctx* c, int species, const double* phi, const dou
   ma.negb = &c->st->negb[species];
   ma.st = c->st;
   cudaError_t e = cudaSuccess;
-  // the Krylov kernel's 4-node group list belongs to the previous domain
-  if (b.qmeta) e = cudaMemsetAsync(b.qmeta, 0, 2 * sizeof(int), c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "init_domain group list reset");
+  ma.qmeta = b.qmeta;
   e = launch_init_domain(ca, ma, c->tile_count, b.ncomp, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "init_domain launch");
   if (c->ncomp_host) {

@@ -74,8 +74,8 @@ struct DevStatus {
   int timeout_site;
   int pad;
   double gersh[2];      // Gershgorin bound of h^2 C per species (max row sum of |h^2 C|)
-  unsigned int barrier; // grid-barrier arrival counter (reset before each cooperative launch)
-  unsigned int pad2;
+  unsigned int barrier; // grid-barrier arrival counter (0 between launches, see barrier_done)
+  unsigned int done;    // CTAs of the running launch that have ended
   int negb[2];          // per species: the beta field has a negative value
   unsigned long long wait_ns;  // limit of every device wait in ns (0: BARRIER_LIMIT_NS)
 };
@@ -97,7 +97,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // Grid-wide barrier for a cooperative launch: a monotonically increasing
-// arrival counter (reset to 0 before the launch).  Barrier number `k`
+// arrival counter (0 at the launch, see barrier_done).  Barrier number `k`
 // (1-based, identical in every CTA) completes when the counter reaches
 // k * gridDim.x.  Ordering: __syncthreads orders the CTA's accesses before
 // thread 0's gpu-scope release add; the waiting thread's gpu-scope acquire
@@ -147,6 +147,25 @@ __device__ __forceinline__ bool grid_barrier(DevStatus* st, unsigned& k, int sit
   __syncthreads();
   return s_ok != 0;
 }
+
+// Last action of every CTA of a cooperative kernel, whatever way it ends: the
+// last CTA to end puts the arrival counter back to 0 for the next launch (a
+// memset before every launch takes 2 to 3 us of the stream's time).  A CTA that
+// ends has polled the counter after its own last arrival, so no arrival is
+// still on its way.
+__device__ __forceinline__ void barrier_done(DevStatus* st) {
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(&st->done, 1u) == gridDim.x - 1u) {
+    st->barrier = 0u;
+    st->done = 0u;
+  }
+}
+
+// barrier_done at every return of a kernel
+struct BarrierDone {
+  DevStatus* st;
+  __device__ __forceinline__ ~BarrierDone() { barrier_done(st); }
+};
 
 // Index of this thread in the node loops: 32-index chunks dealt round-robin
 // over the CTAs (chunk j to warp j / gridDim of CTA j % gridDim), a

@@ -369,7 +369,7 @@ __device__ void metadata_phase(const MetaArgs& a, int ncomp) {
 //            in grid order;
 //   phase 3  (after a second barrier) the row metadata.
 template <int N>
-__global__ void __launch_bounds__(INIT_NT, 1) init_domain_kernel(const ClassifyArgs ca, const MetaArgs ma) {
+__device__ __forceinline__ void init_domain_body(const ClassifyArgs& ca, const MetaArgs& ma) {
   const GridDev& g = ca.g;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   unsigned bar = 0;
@@ -382,6 +382,8 @@ __global__ void __launch_bounds__(INIT_NT, 1) init_domain_kernel(const ClassifyA
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *ma.gersh = 0.0;
     *ma.negb = 0;
+    // the Krylov kernel's 4-node group list belongs to the previous domain
+    if (ma.qmeta) ma.qmeta[0] = ma.qmeta[1] = 0;
   }
   __shared__ int s_w[INIT_NT / 32];
   __shared__ int s_off, s_tot;
@@ -520,6 +522,13 @@ __global__ void __launch_bounds__(INIT_NT, 1) init_domain_kernel(const ClassifyA
   metadata_phase<N>(ma, ncomp);
 }
 
+template <int N>
+__global__ void __launch_bounds__(INIT_NT, 1) init_domain_kernel(const __grid_constant__ ClassifyArgs ca,
+                                                                 const __grid_constant__ MetaArgs ma) {
+  init_domain_body<N>(ca, ma);
+  barrier_done(ca.st);
+}
+
 // ints of scratch the set-up kernel needs: one count per CTA, then two bit
 // planes (computational nodes, signs of phi) of one bit per node
 template <int N>
@@ -547,8 +556,6 @@ cudaError_t launch_init_domain(const ClassifyArgs& ca, const MetaArgs& ma, int* 
   if (e != cudaSuccess) return e;
   if (per < 1) return cudaErrorLaunchOutOfResources;
   const int nb = min(sms, MAX_BLOCKS);
-  e = cudaMemsetAsync(&ca.st->barrier, 0, sizeof(unsigned), stream);
-  if (e != cudaSuccess) return e;
   ClassifyArgs c1 = ca;
   MetaArgs m1 = ma;
   void* args[] = {(void*)&c1, (void*)&m1};

@@ -35,6 +35,7 @@ struct MetaArgs {
   double* bpts;  //   boundary-data coefficient and point (N doubles)
   double* gersh;
   int* negb;
+  int* qmeta;    // nullptr, or the validity flag and length of the group list: zeroed
   DevStatus* st;
 };
 
@@ -97,7 +98,7 @@ struct SpeciesDev {
   int* qidx;
   int* qk;
   // qmeta[0] = 1 when qidx / qk hold the list of the current domain (the
-  // host zeroes it with every domain set-up), qmeta[1] = the list length;
+  // set-up zeroes it for every domain), qmeta[1] = the list length;
   // nullptr: the list is built by every launch
   int* qmeta;
   // caller's source (full grid) and boundary data for this launch: F gains
@@ -157,6 +158,7 @@ struct PhipmArgs {
   double* part;
   DevStatus* st;
   StatsDev* stats;
+  int keep_stats;          // 0: the statistics start anew with this launch
 };
 
 template <typename T>

@@ -47,8 +47,6 @@ cudaError_t launch_phipm(const PhipmArgs<T>& a, int nblocks, cudaStream_t stream
   if (a.g.ndim < 2 || a.g.ndim > 4) return cudaErrorInvalidValue;
   void* fn = v.k.fn[a.g.ndim - 2][adj ? 1 : 0];
   if (nblocks > MAX_SUM_BLOCKS) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(&a.st->barrier, 0, sizeof(unsigned), stream);
-  if (e != cudaSuccess) return e;
   void* args[] = {(void*)&a};
   const size_t dsm = adj ? v.k.adj_smem : 0;
   return cudaLaunchCooperativeKernel(fn, nblocks, v.k.nt, args, dsm, stream);

@@ -1261,7 +1261,6 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
     if (threadIdx.x == 0) c.nquad = c.nq_sp[sidx];
     __syncthreads();
   }
-  // the statistics accumulate over the launches of one step (zeroed by the host)
   if (blockIdx.x == 0 && threadIdx.x == 0) c.trace0 = a.stats ? a.stats->trace_len[sidx] : 0;
   if (threadIdx.x == 0) {
     c.t = 0.0;
@@ -1731,11 +1730,16 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
 // kept apart so that their code adds nothing to the other launches.  NT:
 // threads per CTA (one CTA per SM), which fixes the registers per thread.
 template <typename T, int N, bool ADJ, int NT>
-__global__ void __launch_bounds__(NT, 1) phipm_kernel(const __grid_constant__ PhipmArgs<T> a) {
+__device__ __forceinline__ void phipm_body(const PhipmArgs<T>& a) {
   __shared__ Ctl c;
   unsigned bar = 0;
   int red = 0;
   GridSums gs(a.part);
+  // the statistics accumulate over the launches of one step; block 0 alone
+  // reads and writes them
+  if (blockIdx.x == 0 && a.stats && !a.keep_stats)
+    for (int i = threadIdx.x; i < (int)(sizeof(StatsDev) / sizeof(int)); i += blockDim.x)
+      reinterpret_cast<int*>(a.stats)[i] = 0;
   const GridDev& g = a.g;
   const long long gtid = dealt_tid();
   const long long gthreads = (long long)gridDim.x * blockDim.x;
@@ -1992,6 +1996,12 @@ __global__ void __launch_bounds__(NT, 1) phipm_kernel(const __grid_constant__ Ph
       }
     }
   }
+}
+
+template <typename T, int N, bool ADJ, int NT>
+__global__ void __launch_bounds__(NT, 1) phipm_kernel(const __grid_constant__ PhipmArgs<T> a) {
+  phipm_body<T, N, ADJ, NT>(a);
+  barrier_done(a.st);
 }
 
 // The kernels of one precision and CTA size, for the entries below.

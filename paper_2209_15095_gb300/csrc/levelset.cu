@@ -1100,7 +1100,8 @@ __device__ bool reinitialise(const LsArgs& a, LsCtx& c) {
 }
 
 template <int N>
-__global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const LsArgs a) {
+__global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const __grid_constant__ LsArgs a) {
+  const BarrierDone at_end{a.st};
   const GridDev& g = a.g;
   LsCtx c;
   c.bar = 0;
@@ -1410,8 +1411,6 @@ static cudaError_t launch(const LsArgs& a, cudaStream_t stream) {
   }
   const int nb = ls_blocks(a.g.ndim);
   if (nb <= 0) return cudaErrorLaunchOutOfResources;
-  cudaError_t e = cudaMemsetAsync(&a.st->barrier, 0, sizeof(unsigned), stream);
-  if (e != cudaSuccess) return e;
   void* args[] = {(void*)&a};
   return cudaLaunchCooperativeKernel(fn, nb, LS_NT, args, 0, stream);
 }

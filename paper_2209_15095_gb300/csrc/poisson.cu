@@ -67,7 +67,7 @@ __device__ __forceinline__ double cstencil(const PsPoint<N>& o, const GridDev& g
 }
 
 template <int N>
-__global__ void __launch_bounds__(PS_NT, 1) poisson_kernel(const __grid_constant__ PoissonArgs a) {
+__device__ __forceinline__ void poisson_body(const PoissonArgs& a) {
   const SpeciesDev<double>& S = a.S;
   const GridDev& g = a.g;
   const int ncomp = *S.ncomp;
@@ -201,6 +201,12 @@ __global__ void __launch_bounds__(PS_NT, 1) poisson_kernel(const __grid_constant
   }
 }
 
+template <int N>
+__global__ void __launch_bounds__(PS_NT, 1) poisson_kernel(const __grid_constant__ PoissonArgs a) {
+  poisson_body<N>(a);
+  barrier_done(a.st);
+}
+
 cudaError_t launch_poisson(const PoissonArgs& a, cudaStream_t stream) {
   void* fn;
   switch (a.g.ndim) {
@@ -217,8 +223,6 @@ cudaError_t launch_poisson(const PoissonArgs& a, cudaStream_t stream) {
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, PS_NT, 0);
   if (e != cudaSuccess) return e;
   if (per < 1) return cudaErrorLaunchOutOfResources;
-  e = cudaMemsetAsync(&a.st->barrier, 0, sizeof(unsigned), stream);
-  if (e != cudaSuccess) return e;
   PoissonArgs c = a;
   c.cfac = 1.0 / (a.g.h * a.g.h);
   void* args[] = {(void*)&c};
