@@ -64,6 +64,7 @@ struct etd_ctx {
   double* adj_mu[ADJ_NQ_MAX] = {nullptr};
   double* adj_y[ADJ_NQ_MAX] = {nullptr};
   double* facew = nullptr;
+  void* bface = nullptr;  // face means of species 0's beta field (adjoint contexts)
   int nblocks = 0;
   bool fp32 = false;
   int last_nspecies = 0;
@@ -267,7 +268,9 @@ size_t carve(const GridDev& g, const etd_params& p, char* base, etd_ctx* c) {
       }
     }
     double* fw = cv.take<double>(G * 2 * (size_t)g.ndim);
+    void* bf = f32 ? (void*)cv.take<float>(G * g.ndim) : (void*)cv.take<double>(G * g.ndim);
     if (c) c->facew = fw;
+    if (c) c->bface = bf;
   }
   cv.off = (cv.off + 255) & ~size_t(255);
   return cv.off;
@@ -401,6 +404,7 @@ etd_status run_phipm(etd_ctx* c, int mode, double dt, double* const* u, int spec
   a.st = c->st;
   a.stats = c->stats;
   a.keep_stats = keep_stats ? 1 : 0;
+  a.bface = (all || species == 0) && c->sp[0].beta_field ? (const T*)c->bface : nullptr;
   // the 768-thread FP32 kernel when a species of this launch takes the
   // 4-node groups (its latest known point count; only the speed depends on it)
   bool wide = false;
@@ -570,6 +574,7 @@ etd_status etd_init_domain(etd_ctx* c, int species, const double* phi, const dou
   ma.diag = b.diag;
   ma.diagf = b.diagf;
   ma.facew = species == 0 ? c->facew : nullptr;
+  if (species == 0 && beta_field) (c->fp32 ? (void*&)ma.bfacef : (void*&)ma.bface) = c->bface;
   ma.bco = b.bco;
   ma.bpts = b.bpts;
   ma.gersh = &c->st->gersh[species];
@@ -849,6 +854,7 @@ etd_status etd_adjoint_step(etd_ctx* c, int species, double dt, const double* u_
   a.part = c->part;
   a.grad_params = grad_params;
   a.nq = nquad;
+  for (int d = 0; d < 4; ++d) a.face[d] = c->adj[3 + d];
   for (int i = 0; i < nquad; ++i) {
     a.muq[i] = c->adj_mu[i];
     a.yq[i] = c->adj_y[i];

@@ -66,12 +66,17 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_combine_kernel(const AdjointAr
   block_partials<1>(v, a.part);
 }
 
-// Sums the per-block partials in block order and adds them to grad_params[0].
+// Sums the per-block partials in a fixed order (lane-strided, then a warp tree:
+// one thread's 608 dependent FP64 additions took 25 us) and adds them to
+// grad_params[0].
 __global__ void adjoint_alpha_finish_kernel(const double* part, int nblocks, double* grad_params) {
-  if (threadIdx.x != 0) return;
-  double s = 0.0;
-  for (int b = 0; b < nblocks; ++b) s += part[b];
-  grad_params[0] += s;
+  double s0 = 0.0, s1 = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += 64) {
+    s0 += part[b];
+    if (b + 32 < nblocks) s1 += part[b + 32];
+  }
+  const double s = warp_sum(s0 + s1);
+  if (threadIdx.x == 0) grad_params[0] += s;
 }
 
 cudaError_t launch_adjoint_combine(const AdjointArgs& a, cudaStream_t stream) {
@@ -100,41 +105,38 @@ cudaError_t launch_adjoint_rhs(const AdjointArgs& a, double s1, double s2, doubl
   return cudaGetLastError();
 }
 
+// All quadrature times at once, in two kernels: the weighted sum over i of the
+// face derivative, once per face between computational points (a.face[d] at
+// the lower node: four FP64 instructions per time, which bound the kernel),
+// then one update per node (and one atomic per ghost face).
 template <int N>
-__global__ void __launch_bounds__(ADJ_NT) beta_contract_kernel(const AdjointArgs a, const double* __restrict__ mu,
-                                                              const double* __restrict__ y, double coef,
-                                                              double* grad_beta) {
+__global__ void __launch_bounds__(ADJ_NT) beta_faces_kernel(const AdjointArgs a) {
   const int ncomp = *a.ncomp;
-  const double inv_h2 = 1.0 / (a.g.h * a.g.h);
+  const int nq = a.nq;
   for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < ncomp;
        k += (long long)gridDim.x * blockDim.x) {
     const long long p = a.idx[k];
-    const double mp = mu[p], yp = y[p];
-    double own = 0.0;
+    double f[N];
 #pragma unroll
-    for (int d = 0; d < N; ++d) {
+    for (int d = 0; d < N; ++d) f[d] = 0.0;
+    for (int i = 0; i < nq; ++i) {
+      const double* __restrict__ const mu = a.muq[i];
+      const double* __restrict__ const y = a.yq[i];
+      const double mp = mu[p], yp = y[p], w = a.wq[i];
 #pragma unroll
-      for (int si = 0; si < 2; ++si) {
-        const long long q = p + (si == 0 ? -a.g.stride[d] : a.g.stride[d]);
-        if ((a.kind[q] & 3) == K_COMP) {
-          own += 0.5 * (-(mp - mu[q]) * (yp - y[q]) * inv_h2);
-        } else {
-          const double gw = a.facew[k * (2 * N) + 2 * d + si];
-          const double df = -gw * mp * yp * inv_h2;
-          own += 0.5 * df;
-          atomicAdd(grad_beta + q, coef * (0.5 * df));
-        }
+      for (int d = 0; d < N; ++d) {
+        const long long q = p + a.g.stride[d];
+        f[d] = fma(w, -(mp - mu[q]) * (yp - y[q]), f[d]);
       }
     }
-    grad_beta[p] += coef * own;
+    // (off the computational set the value is not read)
+#pragma unroll
+    for (int d = 0; d < N; ++d) a.face[d][p] = f[d];
   }
 }
 
-// All quadrature times in one pass: per face the weighted sum over i of
-// the face derivative, then one update per node (and one atomic per ghost
-// face).
 template <int N>
-__global__ void __launch_bounds__(ADJ_NT) beta_contract_multi_kernel(const AdjointArgs a, double* grad_beta) {
+__global__ void __launch_bounds__(ADJ_NT) beta_gather_kernel(const AdjointArgs a, double* grad_beta) {
   const int ncomp = *a.ncomp;
   const double inv_h2 = 1.0 / (a.g.h * a.g.h);
   const int nq = a.nq;
@@ -147,16 +149,11 @@ __global__ void __launch_bounds__(ADJ_NT) beta_contract_multi_kernel(const Adjoi
 #pragma unroll
       for (int si = 0; si < 2; ++si) {
         const long long q = p + (si == 0 ? -a.g.stride[d] : a.g.stride[d]);
-        double f = 0.0;
         if ((a.kind[q] & 3) == K_COMP) {
-          for (int i = 0; i < nq; ++i) {
-            const double* mu = a.muq[i];
-            const double* y = a.yq[i];
-            f = fma(a.wq[i], -(mu[p] - mu[q]) * (y[p] - y[q]), f);
-          }
-          own += 0.5 * (f * inv_h2);
+          own += 0.5 * (a.face[d][si == 0 ? q : p] * inv_h2);
         } else {
           const double gw = a.facew[k * (2 * N) + 2 * d + si];
+          double f = 0.0;
           for (int i = 0; i < nq; ++i) f = fma(a.wq[i], -gw * a.muq[i][p] * a.yq[i][p], f);
           const double df = 0.5 * (f * inv_h2);
           own += df;
@@ -168,22 +165,17 @@ __global__ void __launch_bounds__(ADJ_NT) beta_contract_multi_kernel(const Adjoi
   }
 }
 
-cudaError_t launch_beta_contract_multi(const AdjointArgs& a, double* grad_beta, cudaStream_t stream) {
-  switch (a.g.ndim) {
-    case 2: beta_contract_multi_kernel<2><<<ADJ_BLOCKS, ADJ_NT, 0, stream>>>(a, grad_beta); break;
-    case 3: beta_contract_multi_kernel<3><<<ADJ_BLOCKS, ADJ_NT, 0, stream>>>(a, grad_beta); break;
-    case 4: beta_contract_multi_kernel<4><<<ADJ_BLOCKS, ADJ_NT, 0, stream>>>(a, grad_beta); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+template <int N>
+static void beta_contract_launch(const AdjointArgs& a, double* grad_beta, cudaStream_t stream) {
+  beta_faces_kernel<N><<<ADJ_BLOCKS, ADJ_NT, 0, stream>>>(a);
+  beta_gather_kernel<N><<<ADJ_BLOCKS, ADJ_NT, 0, stream>>>(a, grad_beta);
 }
 
-cudaError_t launch_beta_contract(const AdjointArgs& a, const double* mu, const double* y, double coef,
-                                 double* grad_beta, cudaStream_t stream) {
+cudaError_t launch_beta_contract_multi(const AdjointArgs& a, double* grad_beta, cudaStream_t stream) {
   switch (a.g.ndim) {
-    case 2: beta_contract_kernel<2><<<ADJ_BLOCKS, ADJ_NT, 0, stream>>>(a, mu, y, coef, grad_beta); break;
-    case 3: beta_contract_kernel<3><<<ADJ_BLOCKS, ADJ_NT, 0, stream>>>(a, mu, y, coef, grad_beta); break;
-    case 4: beta_contract_kernel<4><<<ADJ_BLOCKS, ADJ_NT, 0, stream>>>(a, mu, y, coef, grad_beta); break;
+    case 2: beta_contract_launch<2>(a, grad_beta, stream); break;
+    case 3: beta_contract_launch<3>(a, grad_beta, stream); break;
+    case 4: beta_contract_launch<4>(a, grad_beta, stream); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

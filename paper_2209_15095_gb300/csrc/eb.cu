@@ -255,7 +255,13 @@ __device__ void metadata_phase(const MetaArgs& a, int ncomp) {
       const long long q = p + s;
       const int iq = ip[d] + (si == 0 ? -1 : 1);
       const double bf = a.beta_field ? 0.5 * (a.beta_field[p] + a.beta_field[q]) : a.beta_c;
-      if (a.beta_field && negative(bf)) *a.negb = 1;
+      if (a.beta_field) {
+        if (negative(bf)) *a.negb = 1;
+        // the face's place: its lower node's
+        const long long fp = (long long)d * g.size + (si == 0 ? q : p);
+        if (a.bface) a.bface[fp] = bf;
+        if (a.bfacef) a.bfacef[fp] = (float)bf;
+      }
       double gw = 0.0;  // 1 - w on a ghost face, 0 on a face to a computational point
       // boundary-data slots of this face: coefficient of u_Gamma in the row
       // (beta_f c / h^2, the ghost value's weight on the boundary point) and

@@ -28,6 +28,10 @@ struct MetaArgs {
   int* ncomp;  // written by the compaction, read by the metadata pass
   const double* beta_field;  // node field or nullptr
   double beta_c;
+  // nullptr, or the face means 0.5 (beta_p + beta_{p + e_d}) of the rows' faces,
+  // axis d at d * grid size (adjoint contexts with a beta field; one of the two)
+  double* bface;
+  float* bfacef;
   double* diag;
   float* diagf;  // nullptr unless FP32 vectors are in use
   double* facew; // nullptr, or per point and face: 1 - w on ghost faces, 0 otherwise
@@ -159,6 +163,7 @@ struct PhipmArgs {
   DevStatus* st;
   StatsDev* stats;
   int keep_stats;          // 0: the statistics start anew with this launch
+  const T* bface;          // face means of sp[0]'s beta field (MetaArgs), or nullptr
 };
 
 template <typename T>
@@ -234,14 +239,12 @@ struct AdjointArgs {
   const double* muq[ADJ_NQ_MAX];
   const double* yq[ADJ_NQ_MAX];
   double wq[ADJ_NQ_MAX];
+  double* face[4];  // scratch: the face derivatives per axis (grid)
 };
 cudaError_t launch_adjoint_combine(const AdjointArgs& a, cudaStream_t stream);
 // v1 = dt F(u_n), v2 = dt (F(u_n) - F(u_{n-1})) scaled by (s1, s2) on the computational set
 cudaError_t launch_adjoint_rhs(const AdjointArgs& a, double s1, double s2, double* v1, double* v2, cudaStream_t stream);
-// grad_beta += coef * d(mu^T C y)/d beta (node field, face mean)
-cudaError_t launch_beta_contract(const AdjointArgs& a, const double* mu, const double* y, double coef,
-                                 double* grad_beta, cudaStream_t stream);
-// grad_beta += sum_i wq[i] d(mu_i^T C y_i)/d beta over the quadrature times (one launch)
+// grad_beta += sum_i wq[i] d(mu_i^T C y_i)/d beta over the quadrature times
 cudaError_t launch_beta_contract_multi(const AdjointArgs& a, double* grad_beta, cudaStream_t stream);
 
 }  // namespace etd

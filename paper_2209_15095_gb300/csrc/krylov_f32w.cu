@@ -6,6 +6,7 @@
 // and at twoball3d (114k points per species) 11% (register spills in the
 // per-point paths), so those keep 512.
 #define ETD_RED_MAX_NT 768
+#define ETD_FACE_MEANS 0
 #include "krylov_impl.cuh"
 
 namespace etd {

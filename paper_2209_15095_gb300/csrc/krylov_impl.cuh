@@ -315,10 +315,17 @@ static __device__ __noinline__ void check_basis(Ctl& c, int p, double tol, const
 }
 
 // ---------------------------------------------------------------------------
+// Whether the unit's per-point paths read the face means of a beta field (the
+// 768-thread unit, for problems on the 4-node groups with a constant beta, does
+// not: that code's registers cost its passes 5%).
+#ifndef ETD_FACE_MEANS
+#define ETD_FACE_MEANS 1
+#endif
 // (A x)_p with A = cfac (beta S - D) (SCALED), or (B x)_p = (A x)_p / cfac.
 template <typename T, int N, bool SCALED = true>
 __device__ __forceinline__ T stencil(const T* __restrict__ x, long long p, const GridDev& g, T Dk,
-                                     const double* __restrict__ bfield, T bc, T cfac) {
+                                     const double* __restrict__ bfield, T bc, T cfac,
+                                     const T* __restrict__ bface = nullptr) {
   const T xp = __ldcg(x + p);
   // the sums start from -0: x + (-0) == x exactly, so the first add is free
   if (bfield == nullptr) {
@@ -327,8 +334,18 @@ __device__ __forceinline__ T stencil(const T* __restrict__ x, long long p, const
     for (int d = 0; d < N; ++d) s += __ldcg(x + p - g.stride[d]) + __ldcg(x + p + g.stride[d]);
     return SCALED ? cfac * (bc * s - Dk * xp) : bc * s - Dk * xp;
   }
-  const double bp = __ldg(bfield + p);
   T s = T(-0.0);
+  if (ETD_FACE_MEANS && bface != nullptr) {  // the same means, computed once per domain
+    const T* __restrict__ const bf = bface + p;
+#pragma unroll
+    for (int d = 0; d < N; ++d) {
+      const long long st = g.stride[d], o = (long long)d * g.size;
+      s += __ldg(bf + o - st) * __ldcg(x + p - st);
+      s += __ldg(bf + o) * __ldcg(x + p + st);
+    }
+    return SCALED ? cfac * (s - Dk * xp) : s - Dk * xp;
+  }
+  const double bp = __ldg(bfield + p);
 #pragma unroll
   for (int d = 0; d < N; ++d) {
     const long long st = g.stride[d];
@@ -1243,6 +1260,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
   const float dint = quad_d_int<T, N>(S);  // the diagonal of the full groups (QK_FULL)
   const double anorm = a.cfac * (*S.gersh);
   const double brk = BREAKDOWN_REL * anorm;
+  const T* const bface = ETD_FACE_MEANS && sidx == 0 ? a.bface : nullptr;
   const int m_max = a.m_max;
   // highest phi index: 2 or 3 (any other value of a.p: 2); 0 for the basis
   // on lambda of the adjoint (V_0 = lambda, written by the set-up)
@@ -1319,21 +1337,21 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
       const T tt = (T)t, th2 = (T)(0.5 * t * t);
       node_loop<1>(gtid, gthreads, ncomp, S.idx, [&](const auto& kk, const auto& pp) {
         if (pp[0] < 0) return;
-        const T ay = stencil<T, N>(S.Yg, pp[0], g, diag_of<T>(S, (int)kk[0]), S.beta_field, bc, cfac);
+        const T ay = stencil<T, N>(S.Yg, pp[0], g, diag_of<T>(S, (int)kk[0]), S.beta_field, bc, cfac, bface);
         const T a1 = __ldcg(S.V1c + kk[0]), a2 = __ldcg(S.V2c + kk[0]), a3 = __ldcg(S.V3c + kk[0]);
         S.W1g[pp[0]] = ay + a1 + tt * a2 + th2 * a3;
       });
       if (!grid_barrier(a.st, bar, 10)) return false;
       node_loop<1>(gtid, gthreads, ncomp, S.idx, [&](const auto& kk, const auto& pp) {
         if (pp[0] < 0) return;
-        const T aw = stencil<T, N>(S.W1g, pp[0], g, diag_of<T>(S, (int)kk[0]), S.beta_field, bc, cfac);
+        const T aw = stencil<T, N>(S.W1g, pp[0], g, diag_of<T>(S, (int)kk[0]), S.beta_field, bc, cfac, bface);
         const T a2 = __ldcg(S.V2c + kk[0]), a3 = __ldcg(S.V3c + kk[0]);
         S.W2g[pp[0]] = aw + a2 + tt * a3;
       });
       if (!grid_barrier(a.st, bar, 16)) return false;
       node_loop<1>(gtid, gthreads, ncomp, S.idx, [&](const auto& kk, const auto& pp) {
         if (pp[0] < 0) return;
-        const T aw = stencil<T, N>(S.W2g, pp[0], g, diag_of<T>(S, (int)kk[0]), S.beta_field, bc, cfac);
+        const T aw = stencil<T, N>(S.W2g, pp[0], g, diag_of<T>(S, (int)kk[0]), S.beta_field, bc, cfac, bface);
         S.V[pp[0]] = aw + __ldcg(S.V3c + kk[0]);
       });
     } else {
@@ -1344,7 +1362,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           if (pp[u] < 0) continue;
-          ay[u] = stencil<T, N>(S.Yg, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac);
+          ay[u] = stencil<T, N>(S.Yg, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac, bface);
           a1[u] = __ldcg(S.V1c + kk[u]);
           a2[u] = __ldcg(S.V2c + kk[u]);
         }
@@ -1360,7 +1378,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           if (pp[u] < 0) continue;
-          aw[u] = stencil<T, N>(S.W1g, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac);
+          aw[u] = stencil<T, N>(S.W1g, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac, bface);
           a2[u] = __ldcg(S.V2c + kk[u]);
         }
 #pragma unroll
@@ -1390,8 +1408,8 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
         for (int u = 0; u < U; ++u) {
           if (pp[u] < 0) continue;
           vv[u] = __ldcg(S.V + pp[u]);
-          zz[u] = zb ? stencil<T, N, false>(S.V, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac)
-                     : stencil<T, N>(S.V, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac);
+          zz[u] = zb ? stencil<T, N, false>(S.V, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac, bface)
+                     : stencil<T, N>(S.V, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac, bface);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -1501,8 +1519,8 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
 #pragma unroll
             for (int u = 0; u < UB; ++u) {
               if (pp[u] < 0) continue;
-              zv[u] = zb ? stencil<T, N, false>(Vj, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac)
-                         : stencil<T, N>(Vj, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac);
+              zv[u] = zb ? stencil<T, N, false>(Vj, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac, bface)
+                         : stencil<T, N>(Vj, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac, bface);
               wv[u] = __ldcg(Vj + pp[u]);
               v1v[u] = __ldcg(V1 + pp[u]);
             }
@@ -1531,6 +1549,14 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
               for (int d = 0; d < N; ++d)
                 s += wval<T>(Zp, V1, V2, p - g.stride[d], ca, cb, cc) + wval<T>(Zp, V1, V2, p + g.stride[d], ca, cb, cc);
               s = bc * s;
+            } else if (ETD_FACE_MEANS && bface != nullptr) {
+#pragma unroll
+              for (int d = 0; d < N; ++d) {
+                const long long st = g.stride[d];
+                const T* const fd = bface + (long long)d * g.size + p;
+                s += __ldg(fd - st) * wval<T>(Zp, V1, V2, p - st, ca, cb, cc);
+                s += __ldg(fd) * wval<T>(Zp, V1, V2, p + st, ca, cb, cc);
+              }
             } else {
               const double bp = __ldg(bf + p);
 #pragma unroll
