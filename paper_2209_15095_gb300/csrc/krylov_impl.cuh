@@ -1512,6 +1512,11 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
           });
           if (!grid_barrier(a.st, bar, 15)) return false;
           // pass B_j: Z_j = A V_j from the stored V_j, and the three sums
+          // (FP64: A being symmetric, h_{j-1,j} is h_{j,j-1}, as in the one-pass form,
+          // instead of a third sum over V_{j-1}. The pass is bound by FP64 issue, 9
+          // instructions a point in 3D instead of 10, and by its loads: one ETD2 step
+          // of a 384^3 ball 24.1 -> 23.0 ms, a phi-combination on a 1001^2 disc 1.76
+          // -> 1.70 ms.)
           Acc<T> d1, d2, d3;
           node_loop<SPLIT_UB<T>>(gtid, gthreads, ncomp, S.idx, [&](const auto& kk, const auto& pp) {
             constexpr int UB = NL_U(kk);
@@ -1522,7 +1527,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
               zv[u] = zb ? stencil<T, N, false>(Vj, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac, bface)
                          : stencil<T, N>(Vj, pp[u], g, diag_of<T>(S, (int)kk[u]), S.beta_field, bc, cfac, bface);
               wv[u] = __ldcg(Vj + pp[u]);
-              v1v[u] = __ldcg(V1 + pp[u]);
+              if (sizeof(T) == 4) v1v[u] = __ldcg(V1 + pp[u]);
             }
 #pragma unroll
             for (int u = 0; u < UB; ++u) {
@@ -1530,7 +1535,7 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
               Zn[pp[u]] = zv[u];
               d1.add(wv[u], wv[u]);
               d2.add(zv[u], wv[u]);
-              d3.add(zv[u], v1v[u]);
+              if (sizeof(T) == 4) d3.add(zv[u], v1v[u]);
             }
           });
           sums[0] = d1.value();
@@ -1589,9 +1594,10 @@ __device__ bool phipm_species(const PhipmArgs<T>& a, const SpeciesDev<T>& S, int
             root_pair(tot[0], hn, rhn);
             const bool bd = __double_as_longlong(hn) < __double_as_longlong(brk);  // both non-negative
             const double sj = bd ? 0.0 : rhn, sp = c.scale[j - 1];
-            // lane 0: h_jj = zfac tot1 sj^2; lane 1: h_{j-1,j} = zfac tot2 sj s_{j-1}
+            // lane 0: h_jj = zfac tot1 sj^2; lane 1: h_{j-1,j} = tot2 sj s_{j-1}, for
+            // zb h_{j,j-1} in its place
             double h = (lane == 0 ? tot[1] : tot[2]) * sj * (lane == 0 ? sj : sp);
-            if (zb) h *= zfac;
+            if (zb) h = lane == 0 ? h * zfac : bd ? 0.0 : hn;
             // coefficients of Z_j (lane 2), V_j (lane 0), V_{j-1} (lane 1)
             const double cf = lane == 2 ? sj * zfac : -h * (lane == 0 ? sj : sp);
             if (lane == 0) {
