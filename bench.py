@@ -514,8 +514,9 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # levelset_kernel<3> on star3d from one ncu capture (command and figures in
 # profiles/levelset_kernel_star3d.md), valid only for the kernel sources whose
 # SHA-256 prefix is recorded here; any change to them reports null.
-LS_TRAFFIC = {"sources": ("levelset.cu", "levelset.cuh", "common.cuh"), "sha256": "a1d876dc469ba6b0",
-              "no_reinit": 22.07e6, "reinit": 22.66e6}
+LS_TRAFFIC = {"sources": ("levelset.cu", "levelset.cuh", "common.cuh", "weno_int.cuh", "int64math.cuh"),
+              "sha256": "18d0e172a060582b",
+              "no_reinit": 24.02e6, "reinit": 24.94e6}
 
 
 def levelset_traffic(reinit_fraction):
@@ -532,8 +533,10 @@ def levelset_traffic(reinit_fraction):
 
 def levelset_flops(info, ndim):
     """Algorithmic FP64 flops of one level-set launch, counted from the
-    formulation the kernel evaluates (add/mul/div/sqrt/min/max 1, fma 2):
-    one Godunov/HJ-WENO5 node-stage costs 106 flops per axis (6 differences,
+    floating-point formulation (add/mul/div/sqrt/min/max 1, fma 2).  The kernel
+    evaluates the derivatives in 64-bit fixed point on the integer pipe; the
+    count is that of the method, so that runs stay comparable.
+    One Godunov/HJ-WENO5 node-stage costs 106 flops per axis (6 differences,
     the Jiang-Peng pair of one-sided derivatives with shared second
     differences and one shared division: 92, the Godunov selection: 4, the
     rest 4) plus 7 per node (square root, 1/h, the RK3 update); the Stefan
@@ -553,7 +556,8 @@ def levelset_flops(info, ndim):
 def roofline(r, w, avg_parts, names):
     """Dominant kernel: the largest share of the step.  The Krylov kernel is
     reported against HBM bandwidth with its algorithmic bytes; the level-set
-    kernel, FP64-ALU bound, against the FP64 rate."""
+    kernel against the FP64 rate its formulas would need (it evaluates the
+    WENO5 derivatives on the integer pipe)."""
     import numpy as np
 
     peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
@@ -575,7 +579,7 @@ def roofline(r, w, avg_parts, names):
     ls = {"bound": "alu", "kernel": names[0], "achieved": flops / t_ls / 1e12, "peak": FP64_PEAK_TFLOPS,
           "unit": "TFLOP/s", "frac": flops / t_ls / 1e12 / FP64_PEAK_TFLOPS,
           "traffic": levelset_traffic(r["reinit_steps"] / steps) if w.name == "star3d" else None,
-          "peak_source": "FP64 nominal: 152 SMs x 2 FMA/clk x 2 flop x 2.07 GHz (unit counts and clock); the measured FP64 FMA rate on this GB300 is 1.005 TFLOP/s",
+          "peak_source": "FP64 nominal: 152 SMs x 2 FMA/clk x 2 flop x 2.07 GHz (unit counts and clock); the measured FP64 FMA rate on this GB300 is 1.005 TFLOP/s; the WENO5 derivatives run on the integer pipe in 64-bit fixed point",
           "algorithmic_flops_per_launch": flops}
     out = ls if dom == 0 else krylov
     out = dict(out)
@@ -702,19 +706,19 @@ def krylov_fp64_ops(ncomp, iters, subs):
     large problem (split passes), as the kernel formulates the method: the
     ETD2 set-up 8 per point; per substep the w_1 pass 10 (7-point stencil 8,
     two terms), the w_2 pass 9, P_0 9 (stencil on B = A / cfac 7, two sums),
-    per Krylov vector 13 (V_j = ca Z + cb V_{j-1} + cc V_{j-2}: 3; Z = B V_j:
-    7; three sums), and the combination m + 3."""
-    return ncomp * (8 + subs * 31 + iters * 14)
+    per Krylov vector 12 (V_j = ca Z + cb V_{j-1} + cc V_{j-2}: 3; Z = B V_j:
+    7; two sums), and the combination m + 3."""
+    return ncomp * (8 + subs * 31 + iters * 13)
 
 
 def krylov_bytes_two_pass(ncomp, iters, subs, s):
     """Algorithmic bytes with the two passes per Krylov vector that large FP64
-    problems run (7s + b per point and vector: pass A reads Z_{j-1}, V_{j-1},
-    V_{j-2} and writes V_j; pass B reads V_j, V_{j-1}, writes Z_j), the rest
+    problems run (6s + b per point and vector: pass A reads Z_{j-1}, V_{j-1},
+    V_{j-2} and writes V_j; pass B reads V_j, writes Z_j), the rest
     as krylov_bytes.  Large FP32 problems run one pass per vector (read
     u_{j-1}, V_{j-1}, write V_j, u_j), within krylov_bytes' count."""
     b = (8.0 if s == 8 else 4.0) + 4.0
-    return ncomp * (iters * (7 * s + b) + subs * 2 * (3 * s + b) + (iters + 2 * subs) * s + subs * 16 + 48)
+    return ncomp * (iters * (6 * s + b) + subs * 2 * (3 * s + b) + (iters + 2 * subs) * s + subs * 16 + 48)
 
 
 def run_stress(etd, stream, dev, steps, n=512, precisions="both"):
@@ -820,7 +824,7 @@ def run_poisson(etd, stream, dev, N=1280):
     return {"workload": "virus2d", "N": N, "ncomp": nc, "cg_iters": it, "rel_resid": res, "ms": ms,
             "mcell_iters_per_s": nc * it / (ms / 1e3) / 1e6, "achieved_gbs": bytes_ / (ms / 1e3) / 1e9,
             "frac_of_hbm": bytes_ / (ms / 1e3) / 1e9 / hbm, "max_err_vs_exact": err,
-            "note": "FP64 conjugate gradients, one persistent kernel with 3 grid barriers per iteration"}
+            "note": "FP64 conjugate gradients, one persistent kernel with 2 grid barriers per iteration"}
 
 
 def run_e2e(args, w, make_ctx, initial_state, one_step, stream, flush, dev):
