@@ -89,6 +89,22 @@ ETD_HD u64 normalise(U128 s, int& z) {
   return (u64)shfl32(b, a, n) << 32 | shfl32(c, b, n);
 }
 
+// A single-precision seed of a value in (1, 2] as r 2^31, 1 <= r < 2: the
+// exponent is dropped, so a seed that ends outside [1, 2) would enter at half
+// or twice its value.  The approximations' documented errors (1 ulp of the
+// reciprocal, 2^-22.9 of the reciprocal root) allow both sides; a seed moved
+// onto the end is within those errors.
+ETD_HD unsigned seed_bits(float r) {
+  r = fminf(fmaxf(r, 1.0f), 1.9999998f);
+#ifdef __CUDA_ARCH__
+  const unsigned b = __float_as_uint(r);
+#else
+  unsigned b;
+  memcpy(&b, &r, 4);
+#endif
+  return (b & 0x7fffffu) << 8 | 0x80000000u;
+}
+
 // Reciprocal root and root of x = M 2^-64, 1/4 <= x < 1: r 2^63 and sqrt(x) 2^63,
 // to about 2^-60: a single-precision reciprocal root r0, then r = r0 (1 + e/2 +
 // 3 e^2 / 8) with e = 1 - x r0^2 (|e| < 2^-21), sqrt(x) = x r.
@@ -99,16 +115,11 @@ ETD_HD void root_u(u64 M, u64& r, u64& gx) {
 #ifdef __CUDA_ARCH__
   f = __uint_as_float(fb);
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
-  rf = fminf(rf, 1.9999998f);
-  const unsigned rb = __float_as_uint(rf);
 #else
   memcpy(&f, &fb, 4);
   rf = 1.0f / sqrtf(f);
-  if (rf > 1.9999998f) rf = 1.9999998f;
-  unsigned rb;
-  memcpy(&rb, &rf, 4);
 #endif
-  const unsigned r0 = (rb & 0x7fffffu) << 8 | 0x80000000u;  // (1, 2) 2^31
+  const unsigned r0 = seed_bits(rf);
   const i64 e = (i64)((1ull << 62) - mulhi_u(M, wide(r0, r0)));  // e 2^62
   const int eh = (int)(e >> 16);
   const i64 e1 = (e >> 1) + ((i64)eh * eh * 3 >> 33);

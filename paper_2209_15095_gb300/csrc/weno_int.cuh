@@ -85,22 +85,16 @@ ETD_HD i64 to_fix(double f, int eh) {
 // e = 1 - w r0 (|e| < 2^-21).
 ETD_HD u64 recip_u(u64 w) {
   const unsigned wh = hi32(w);
-  float f;
-  unsigned fb = 0x3f000000u | ((wh - 0x40000000u) >> 7);  // w 2^-63, truncated
+  float f, rf;
+  const unsigned fb = 0x3f000000u | ((wh - 0x40000000u) >> 7);  // w 2^-63, truncated
 #ifdef __CUDA_ARCH__
   f = __uint_as_float(fb);
-  float rf;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
-  rf = fminf(rf, 1.9999998f);
-  const unsigned r0 = (__float_as_uint(rf) & 0x7fffffu) << 8 | 0x80000000u;  // (1, 2) 2^31
 #else
   memcpy(&f, &fb, 4);
-  float rf = 1.0f / f;
-  if (rf > 1.9999998f) rf = 1.9999998f;
-  unsigned rb;
-  memcpy(&rb, &rf, 4);
-  const unsigned r0 = (rb & 0x7fffffu) << 8 | 0x80000000u;
+  rf = 1.0f / f;
 #endif
+  const unsigned r0 = seed_bits(rf);
   // w r0 2^-32, about 2^62: p = w r0 >> 32 as 64 bits
   const u64 p = wide(hi32(w), r0, wide(lo32(w), r0) >> 32);
   const i64 e = (i64)((1ull << 62) - p);  // e 2^62, |e| < 2^42
