@@ -240,7 +240,7 @@ __device__ __forceinline__ float* stage_f32(const LsArgs& a, int k) {
 enum : int { COPY_INT = 1, COPY_F32 = 2 };
 __device__ __forceinline__ void stage_put(const LsArgs& a, int copies, int k, long long p, double v) {
   stage_f64(a, k)[p] = v;
-  if (copies & COPY_INT) stage_int(a, k)[p] = to_fix(v, a.wi.eh);
+  if (copies & COPY_INT) stage_int(a, k)[p] = to_fix(v, a.wi.eh, FIX_KMAX);
   if (copies & COPY_F32) stage_f32(a, k)[p] = to_f32_rn(v);
 }
 
@@ -276,16 +276,15 @@ __device__ __forceinline__ double grad_int(const LsArgs& a, const StageLane<N>& 
 #pragma unroll
     for (int k = -3; k <= 3; ++k) F[d][k + 3] = k == 0 ? own : __ldcg(src + e.p + step_of<N>(g, e, d, k));
   }
-  const int oh = (int)hi32((u64)own);
-  bool ok = (unsigned)(oh ^ (oh >> 31)) < FIX_OWN_HI;
+  unsigned big = 0;
   U128 acc{0, 0};
 #pragma unroll
   for (int d = 0; d < N; ++d) {
-    i64 mx;
-    ok = weno_axis(F[d], positive, a.wi, mx) && ok;
-    acc = add128(acc, sq128(mx));
+    i64 q[6];
+    big |= fix_diffs(F[d], q);
+    acc = add128(acc, sq128(weno_axis(q, positive, a.wi)));
   }
-  if (ok) return grad_of(acc, a.wi);
+  if (big < FIX_DIFF_HI && hi_mag(own) < FIX_OWN_HI) return grad_of(acc, a.wi);
   double s = 0.0;
   for (int d = 0; d < N; ++d) {
     double f[7];
@@ -305,12 +304,11 @@ __device__ __forceinline__ double grad_int_split(const LsArgs& a, const StageLan
   U128 sq{0, 0};
   bool ok = true;
   if (e.p >= 0) {
-    i64 F[7], mx;
+    i64 F[7], q[6];
 #pragma unroll
     for (int k = -3; k <= 3; ++k) F[k + 3] = __ldcg(src + e.p + step_of<N>(g, e, e.ax, k));
-    const int oh = (int)hi32((u64)F[3]);
-    ok = weno_axis(F, positive, a.wi, mx) && (unsigned)(oh ^ (oh >> 31)) < FIX_OWN_HI;
-    sq = sq128(mx);
+    ok = fix_diffs(F, q) < FIX_DIFF_HI && hi_mag(F[3]) < FIX_OWN_HI;
+    sq = sq128(weno_axis(q, positive, a.wi));
   }
   const int base = (int)(threadIdx.x & 31) - e.ax;
   U128 acc{0, 0};
@@ -1048,7 +1046,7 @@ __device__ __forceinline__ void stage_init(const LsArgs& a, int copies, long lon
   a.b.p1[p] = v;
   a.b.p2[p] = v;
   if (copies & COPY_INT) {
-    const i64 f = to_fix(v, a.wi.eh);
+    const i64 f = to_fix(v, a.wi.eh, FIX_KMAX);
 #pragma unroll
     for (int k = 0; k < 3; ++k) stage_int(a, k)[p] = f;
   }

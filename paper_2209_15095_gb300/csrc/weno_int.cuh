@@ -13,9 +13,12 @@
 //     squares, pairwise products and the quotient 64-bit mantissas: the
 //     weights carry an error below 2^-53, against about 20 roundings of
 //     2^-53 in the FP64 form, and the result one of a few units.
-// The arithmetic covers |phi| < 16 2^floor(log2 h) (at least 8h; the tube's
-// phi is at most 6h + one node) with adjacent differences below 2^57 units
-// (at least 4h); other nodes take the FP64 form (weno_in_range).
+// Only differences enter the arithmetic: it covers adjacent differences in
+// [-2^57, 2^57) units (at least 4h) of values below 2^61 units (at least 64h,
+// FIX_KMAX; where phi is not clamped, the stencil of a tube node reaches 10h).
+// Other nodes take the FP64 form as well.  With values limited to 2^58 units (8h
+// to 16h) 91% of the warps of a 200^3 grid with an unclamped phi took both: an
+// advancing launch 1430 us, a reinitialising one 16.4 ms, against 870 us and 3.77 ms.
 #pragma once
 #include "int64math.cuh"
 
@@ -29,7 +32,8 @@ struct WenoInt {
 };
 
 constexpr i64 FIX_OUT = 1ll << 62;  // stored for a value out of range (either sign)
-constexpr unsigned FIX_OWN_HI = 1u << 26;   // |F| < 2^58
+constexpr int FIX_KMAX = 6;                 // the stages take |phi| < 2^7 2^eh
+constexpr unsigned FIX_OWN_HI = 1u << 29;   // |F| < 2^61
 constexpr unsigned FIX_DIFF_HI = 1u << 25;  // |difference| < 2^57
 
 inline WenoInt weno_int(double h, double eps) {
@@ -62,8 +66,8 @@ inline WenoInt weno_int(double h, double eps) {
 }
 
 // phi 2^S as a 64-bit integer, to nearest; FIX_OUT with phi's sign when
-// |phi| >= 16 2^eh, infinite or NaN.
-ETD_HD i64 to_fix(double f, int eh) {
+// |phi| >= 2^(kmax + 1) 2^eh (kmax <= FIX_KMAX), infinite or NaN.
+ETD_HD i64 to_fix(double f, int eh, int kmax = 3) {
 #ifdef __CUDA_ARCH__
   const u64 b = (u64)__double_as_longlong(f);
 #else
@@ -72,12 +76,33 @@ ETD_HD i64 to_fix(double f, int eh) {
 #endif
   const int k = (int)((b >> 52) & 0x7ff) - 1023 - eh;
   const i64 sg = (i64)b >> 63;
-  if (k > 3) return (FIX_OUT ^ sg) - sg;
-  const int r = 4 - k;  // the mantissa times 2^6, shifted right by r >= 1
-  if (r > 60) return 0;
-  const u64 m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 6;
+  if (k > kmax) return (FIX_OUT ^ sg) - sg;
+  const int r = 7 - k;  // the mantissa times 2^9, shifted right by r >= 1
+  if (r > 62) return 0;
+  const u64 m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 9;
   const i64 v = (i64)((m + (1ull << (r - 1))) >> r);
   return (v ^ sg) - sg;
+}
+
+// |x| as far as its upper word decides: the word, complemented if negative
+ETD_HD unsigned hi_mag(i64 x) {
+  const int h = (int)hi32((u64)x);
+  return (unsigned)(h ^ (h >> 31));
+}
+// The six differences of seven values; returns a bound of their magnitudes, which
+// the integer form takes below FIX_DIFF_HI.  A value out of range (FIX_OUT)
+// differs by 2^61 or more from every one in range and from FIX_OUT of the other
+// sign: beside a node's own value (FIX_OWN_HI) the differences decide.
+ETD_HD unsigned fix_diffs(const i64 (&F)[7], i64 (&q)[6]) {
+  unsigned big = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int i = 0; i < 6; ++i) {
+    q[i] = (i64)((u64)F[i + 1] - (u64)F[i]);
+    big |= hi_mag(q[i]);
+  }
+  return big;
 }
 
 // 2^126 / w for w in [2^62, 2^63), to about 2^-58: a single-precision
@@ -153,8 +178,8 @@ ETD_HD i64 weno_phi12(i64 a, i64 b, i64 c, i64 d, const WenoInt& k) {
 }
 
 // max(d, 0)-style upwind value of one axis, 12 max(d-, -d+, 0) for outward
-// motion (positive) or its mirror image, from the seven values F (units
-// 2^-S); false if a difference is out of range.  Only one side's weights are
+// motion (positive) or its mirror image, from the six differences q (units
+// 2^-S; of no use where they are out of range).  Only one side's weights are
 // evaluated: the larger of the two candidates a, b is decided on a
 // single-precision estimate of a - b = +-(d- + d+), whose error stays below
 // `tol` (the second differences enter truncated to 2^-22 2^eh, which moves a
@@ -163,16 +188,9 @@ ETD_HD i64 weno_phi12(i64 a, i64 b, i64 c, i64 d, const WenoInt& k) {
 // not decide, both sides are evaluated.  Equal values (all second
 // differences 0) need no decision.
 #ifdef __CUDACC__
-__device__ __forceinline__ bool weno_axis(const i64 (&F)[7], bool positive, const WenoInt& k, i64& out) {
+__device__ __forceinline__ i64 weno_axis(const i64 (&q)[6], bool positive, const WenoInt& k) {
   const float epsf = k.epsf;
-  i64 q[6], e[5];
-  unsigned big = 0;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    q[i] = F[i + 1] - F[i];
-    const int h = (int)hi32((u64)q[i]);
-    big |= (unsigned)(h ^ (h >> 31));
-  }
+  i64 e[5];
 #pragma unroll
   for (int i = 0; i < 5; ++i) e[i] = q[i + 1] - q[i];
   const i64 cen = 7 * (q[2] + q[3]) - (q[1] + q[4]);
@@ -209,8 +227,7 @@ __device__ __forceinline__ bool weno_axis(const i64 (&F)[7], bool positive, cons
     both = false;
     minus = !minus;
   }
-  out = best;
-  return big < FIX_DIFF_HI;
+  return best;
 }
 #endif
 
