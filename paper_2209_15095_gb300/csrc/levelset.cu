@@ -213,17 +213,6 @@ __device__ __forceinline__ C weno5_upwind(const Weno5Terms<C>& t, C r0, C r1, bo
   return max0(positive ? dm : -dm, positive ? -dp : dp);
 }
 
-// One axis of the Godunov |grad phi|, scaled by 12, in FP64: the form for
-// values out of the integer form's range (weno_int.cuh), h 12 |.| from
-// undivided differences with eps' = 4 eps h^2.
-__device__ __noinline__ double godunov_mx_f64(const double* f, bool positive, double h) {
-  double q[6];
-#pragma unroll
-  for (int k = 0; k < 6; ++k) q[k] = f[k + 1] - f[k];
-  const Weno5Terms<double> t = weno5_terms<double>(q, 4.0 * WENO_EPS * h * h);
-  return weno5_upwind<double>(t, 4.0 / t.W[0], 4.0 / t.W[1], positive);
-}
-
 // The values of phi, p_1 and p_2 (k = 0, 1, 2) as the stages' stencils read
 // them: FP64, 64-bit integers (weno_int.cuh) and FP32.  A value is converted
 // once, where it is written, instead of at each of the 6N + 1 nodes that
@@ -263,8 +252,41 @@ __device__ __forceinline__ long long step_of(const GridDev& g, const StageLane<N
   return (long long)(i - e.ix[d]) * g.stride[d];
 }
 
+// Axis d (index i along it) of the Godunov |grad phi| at a node, scaled by 12 h,
+// where the integer form's values or differences leave their range
+// (weno_int.cuh): from the integer copy in larger units, or, with values out of
+// range, in FP64 from undivided differences with eps' = 4 eps h^2.  Out of line:
+// few nodes take it, and its code inside the stages costs them 0.4%.
+__device__ __noinline__ double godunov_mx_far(const LsArgs& a, int p, int i, int d, const i64* __restrict__ src,
+                                              const double* __restrict__ dsrc, bool positive) {
+  const GridDev& g = a.g;
+  i64 F[7], q[6];
+  unsigned top = 0;
+  const auto at = [&](int k) { return p + (long long)(min(max(i + k, 0), g.n[d] - 1) - i) * g.stride[d]; };
+#pragma unroll
+  for (int k = -3; k <= 3; ++k) {
+    F[k + 3] = __ldcg(src + at(k));
+    top |= hi_mag(F[k + 3]);
+  }
+  const unsigned big = fix_diffs(F, q);
+  if (top < FIX_OWN_HI) return weno_steep12(q, big, positive, a.wi);
+  double f[7], qd[6];
+#pragma unroll
+  for (int k = -3; k <= 3; ++k) f[k + 3] = __ldcg(dsrc + at(k));
+#pragma unroll
+  for (int k = 0; k < 6; ++k) qd[k] = f[k + 1] - f[k];
+  const Weno5Terms<double> t = weno5_terms<double>(qd, 4.0 * WENO_EPS * g.h * g.h);
+  // one division where the product stays within the exponent range
+  const double D = t.W[0] * t.W[1];
+  if (((unsigned)__double2hiint(D) >> 20) - 23u < 2000u) {
+    const double r = 4.0 / D;
+    return weno5_upwind<double>(t, t.W[1] * r, t.W[0] * r, positive);
+  }
+  return weno5_upwind<double>(t, 4.0 / t.W[0], 4.0 / t.W[1], positive);
+}
+
 // |grad phi| (Godunov, WENO5) at a node from the integer copy `src`; out of
-// range: in FP64 from `dsrc`.
+// range: an axis at a time (godunov_mx_far).
 template <int N>
 __device__ __forceinline__ double grad_int(const LsArgs& a, const StageLane<N>& e, const i64* __restrict__ src,
                                            const double* __restrict__ dsrc, bool positive) {
@@ -286,10 +308,9 @@ __device__ __forceinline__ double grad_int(const LsArgs& a, const StageLane<N>& 
   }
   if (big < FIX_DIFF_HI && hi_mag(own) < FIX_OWN_HI) return grad_of(acc, a.wi);
   double s = 0.0;
+#pragma unroll
   for (int d = 0; d < N; ++d) {
-    double f[7];
-    for (int k = -3; k <= 3; ++k) f[k + 3] = __ldcg(dsrc + e.p + step_of<N>(g, e, d, k));
-    const double mx = godunov_mx_f64(f, positive, g.h);
+    const double mx = godunov_mx_far(a, e.p, e.ix[d], d, src, dsrc, positive);
     s = fma(mx, mx, s);
   }
   return sqrt(s) * a.inv_h12;
@@ -321,12 +342,10 @@ __device__ __forceinline__ double grad_int_split(const LsArgs& a, const StageLan
   }
   double gr = grad_of(acc, a.wi);
   if (__any_sync(0xffffffffu, !all)) {
-    double m = 0.0;
-    if (e.p >= 0) {
-      double f[7];
-      for (int k = -3; k <= 3; ++k) f[k + 3] = __ldcg(dsrc + e.p + step_of<N>(g, e, e.ax, k));
-      m = godunov_mx_f64(f, positive, g.h);
-    }
+    int i = e.ix[0];
+#pragma unroll
+    for (int d = 1; d < N; ++d) i = e.ax == d ? e.ix[d] : i;
+    const double m = e.p >= 0 ? godunov_mx_far(a, e.p, i, e.ax, src, dsrc, positive) : 0.0;
     double s = 0.0;
 #pragma unroll
     for (int d = 0; d < N; ++d) {
@@ -943,8 +962,8 @@ __device__ __forceinline__ void stage_push(const LsArgs& a, int i, bool front) {
 // CTAs (every SM gets its share of each kind).  Front entries go a lane each,
 // or, where they then still make one round of the warps at most, an axis per
 // lane (32 / N entries per warp): the same instructions in all, a third (3D) of
-// the dependent chain per warp.  Back entries go a lane each, before and after
-// that round, and do not count: a reinitialisation of the mixed variant, with few
+// the dependent chain per warp.  Back entries go a lane each in what rounds
+// follow, and do not count: a reinitialisation of the mixed variant, with few
 // front entries among many, took 1.71 instead of 1.35 ms on a steep phi at 200^3 where
 // they did (five steps of the 4D ellipsoid at 48^4 3.66 instead of 3.42 ms).
 template <int N>

@@ -16,7 +16,8 @@
 // Only differences enter the arithmetic: it covers adjacent differences in
 // [-2^57, 2^57) units (at least 4h) of values below 2^61 units (at least 64h,
 // FIX_KMAX; where phi is not clamped, the stencil of a tube node reaches 10h).
-// Other nodes take the FP64 form as well.  With values limited to 2^58 units (8h
+// Axes with larger differences go through the same arithmetic in larger units
+// (weno_steep12), values out of range through the FP64 form.  With values limited to 2^58 units (8h
 // to 16h) 91% of the warps of a 200^3 grid with an unclamped phi took both: an
 // advancing launch 1430 us, a reinitialising one 16.4 ms, against 870 us and 3.77 ms.
 #pragma once
@@ -27,6 +28,7 @@ namespace etd {
 struct WenoInt {
   int eh;            // floor(log2 h)
   u64 e4hi, e4lo;    // (3/4) eps' 2^2S = 3e-6 (h 2^S)^2, 128 bits
+  double unit;       // 2^-S
   double scale;      // 2^-S / (12 h): the gradient from 12 times itself in units
   float epsf;        // (3/4) eps' in units of 2^eh, squared
 };
@@ -44,6 +46,7 @@ inline WenoInt weno_int(double h, double eps) {
   if (w.eh < -900 || w.eh > 900) {  // near the ends of the exponent range: nothing is in range
     w.eh = -4000;
     w.e4hi = w.e4lo = 0;
+    w.unit = 0.0;
     w.scale = 0.0;
     w.epsf = 0.f;
     return w;
@@ -61,6 +64,7 @@ inline WenoInt weno_int(double h, double eps) {
   const u64 sb = (u64)(1023 + w.eh - 54) << 52;
   double s;
   memcpy(&s, &sb, 8);  // 2^-S
+  w.unit = s;
   w.scale = s / (12.0 * h);
   return w;
 }
@@ -184,14 +188,15 @@ ETD_HD i64 weno_phi12(i64 a, i64 b, i64 c, i64 d, const WenoInt& k) {
 // single-precision estimate of a - b = +-(d- + d+), whose error stays below
 // `tol` (the second differences enter truncated to 2^-22 2^eh, which moves a
 // weight by up to 0.3%: 5.1 2^-22 / sqrt(3e-6) per s_k, four-fold in the
-// quotient, rounded up to 2^-7 of the terms it multiplies); where that does
-// not decide, both sides are evaluated.  Equal values (all second
+// quotient, rounded up to tolf = 2^-7 of the terms it multiplies); where that
+// does not decide, both sides are evaluated.  Equal values (all second
 // differences 0) need no decision.
-#ifdef __CUDACC__
-__device__ __forceinline__ i64 weno_axis(const i64 (&q)[6], bool positive, const WenoInt& k) {
+ETD_HD i64 weno_axis(const i64 (&q)[6], bool positive, const WenoInt& k, float tolf = 0x1p-7f) {
   const float epsf = k.epsf;
   i64 e[5];
+#ifdef __CUDA_ARCH__
 #pragma unroll
+#endif
   for (int i = 0; i < 5; ++i) e[i] = q[i + 1] - q[i];
   const i64 cen = 7 * (q[2] + q[3]) - (q[1] + q[4]);
   // the estimate, in units of 2^eh (f = 2^-22 leading words)
@@ -210,10 +215,14 @@ __device__ __forceinline__ i64 weno_axis(const i64 (&q)[6], bool positive, const
   const auto phi = [](float s0, float s1, float s2, float X, float Yv) {
     const float d0 = s0 * s0, d1 = s1 * s1, d2 = s2 * s2;
     const float A = d1 * d2, AB = fmaf(6.f, d0 * d2, A), C3 = 3.f * (d0 * d1);
+#ifdef __CUDA_ARCH__
     return __fdividef(fmaf(4.f * A, X, (C3 - AB) * Yv), AB + C3);
+#else
+    return fmaf(4.f * A, X, (C3 - AB) * Yv) / (AB + C3);
+#endif
   };
   const float D = 2.f * ((float)(int)hi32((u64)cen) * 0x1p-22f) - phi(m0, m1, m2, X0, Y) + phi(p0, p1, p2, X1, Y);
-  const float tol = fmaf(0x1p-7f, 4.f * (fabsf(X0) + fabsf(X1)) + 2.f * fabsf(Y), 0x1p-14f);
+  const float tol = fmaf(tolf, 4.f * (fabsf(X0) + fabsf(X1)) + 2.f * fabsf(Y), 0x1p-14f);
   const bool flat = (e[0] | e[1] | e[2] | e[3] | e[4]) == 0;  // d- = d+ = cen / 12
   bool minus = (flat ? cen > 0 : D > 0.f) == positive;
   bool both = !flat && !(fabsf(D) > tol);
@@ -229,7 +238,35 @@ __device__ __forceinline__ i64 weno_axis(const i64 (&q)[6], bool positive, const
   }
   return best;
 }
-#endif
+
+// 12 h max(d-, -d+, 0) or its mirror image where the differences (bound `big`,
+// fix_diffs) of values in range may leave weno_axis's range: the same in units
+// 2^(s-S) in which they fit, so that they are rounded by 2^-57 of the largest at
+// most (eps' enters the side's estimate smaller by 2^2s, its truncation 2^s times
+// as large): an error below the FP64 form's, but beside a kink that only the
+// stencil's far end sees (to 1e-15 of the gradient), and a call's result is as far
+// from extended precision as with the FP64 form.  Such nodes are those of a phi
+// far from a distance, until it is reinitialised, and their neighbours.  Steps on
+// phi = slope (r - R) in 3D, with the FP64 form after the integer one for such
+// nodes / with this / with the FP64 form alone: slope 9 at 200^3 952 / 625 / 782 us,
+// slope 20 at 160^3 685 / 447 / 594 us, with reinitialisation at 200^3, slope 3 7.66 /
+// 3.85 / 6.60 ms, slope 9 5.12 / 3.18 / 3.95 ms.
+ETD_HD double weno_steep12(i64 (&q)[6], unsigned big, bool positive, const WenoInt& k) {
+  const int z = clz32(big);
+  const int s = z < 7 ? 7 - z : 0;  // |q| 2^-s < 2^57; s <= 5 (values in range: z >= 2)
+  if (s > 0) {
+    const i64 half = 1ll << (s - 1);
+    for (int i = 0; i < 6; ++i) q[i] = (q[i] + half) >> s;
+  }
+  WenoInt ks = k;
+  const float f = (float)(1 << s);
+  if (s > 0) {
+    ks.e4lo = k.e4lo >> (2 * s) | k.e4hi << (64 - 2 * s);
+    ks.e4hi = k.e4hi >> (2 * s);
+    ks.epsf = k.epsf / (f * f);
+  }
+  return (double)weno_axis(q, positive, ks, 0x1p-7f * f) * (k.unit * (double)(1 << s));
+}
 
 // sqrt(acc) 2^-S / (12 h) as a double: acc = x 2^(128 - z), 1/4 <= x < 1, the
 // root rounded to 53 bits.
