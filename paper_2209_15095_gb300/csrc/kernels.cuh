@@ -175,13 +175,11 @@ constexpr int QUAD_MIN_POINTS = 1 << 18;
 int phipm_max_blocks(int ndim, bool fp32);
 // The Krylov kernels of one precision and CTA size (krylov_impl.cuh):
 // fn[ndim - 2][adjoint instantiation], threads per CTA, the adjoint
-// instantiation's dynamic shared memory, and the loader of the unit's
-// constant table.
+// instantiation's dynamic shared memory.
 struct PhipmKernels {
   void* fn[3][2];
   int nt;
   size_t adj_smem;
-  cudaError_t (*load_consts)();
 };
 
 // Embedded-boundary Poisson solve by conjugate gradients (FP64)

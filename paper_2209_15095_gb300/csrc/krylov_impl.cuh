@@ -36,6 +36,7 @@
 // launches it.  A unit may define ETD_RED_MAX_NT (the block-reduction width)
 // before including it.
 #pragma once
+#include "cheb.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -59,53 +60,8 @@ constexpr int SPLIT_U = sizeof(T) == 8 ? 2 : 4;
 template <typename T>
 constexpr int SPLIT_UB = sizeof(T) == 8 ? 2 : 3;  // the stencil pass (register bound)
 
-// Chebyshev coefficients 2 e^-a I_k(a) of e^(a (x - 1)) for a = 2^(i/2),
-// i = 0 .. CHEB_TABLES - 1, down to 1e-24: table i at c_cheb + c_cheb_at[i]
-// (20 coefficients at a = 1, 87 at 64, 233 at 512).  Each translation unit
-// that instantiates the kernel has its own copy (filled by load_cheb before
-// its first launch).
-constexpr int CHEB_TABLES = 19, CHEB_MAX = 1800;
-static __constant__ double c_cheb[CHEB_MAX];
-static __constant__ double c_cheb_2a[CHEB_TABLES];  // 2 / a
-static __constant__ int c_cheb_at[CHEB_TABLES + 1];
-
-// I_k(a) up to a factor by Miller's downward recurrence I_{k-1} = I_{k+1} +
-// (2k/a) I_k (Abramowitz & Stegun 9.12), normalised by I_0 + 2 sum I_k = e^a.
-static cudaError_t load_cheb() {
-  double tab[CHEB_MAX], two_a[CHEB_TABLES];
-  int at[CHEB_TABLES + 1];
-  int n = 0;
-  for (int i = 0; i < CHEB_TABLES; ++i) {
-    const double a = pow(2.0, 0.5 * i);
-    two_a[i] = 2.0 / a;
-    at[i] = n;
-    double t[512];
-    double up = 0.0, sum = 0.0, cur = 1e-200;
-    for (int k = 511; k >= 0; --k) {  // cur = I_k, up = I_{k+1}
-      t[k] = cur;
-      sum += k > 0 ? 2.0 * cur : cur;
-      const double down = up + 2.0 * k / a * cur;
-      up = cur;
-      cur = down;
-      if (cur > 1e200) {
-        for (int j = k; j < 512; ++j) t[j] *= 1e-200;
-        cur *= 1e-200;
-        up *= 1e-200;
-        sum *= 1e-200;
-      }
-    }
-    for (int k = 0; k < 512 && n < CHEB_MAX; ++k) {
-      const double c = 2.0 * t[k] / sum;
-      if (c < 1e-24) break;
-      tab[n++] = c;
-    }
-  }
-  at[CHEB_TABLES] = n;
-  cudaError_t e = cudaMemcpyToSymbol(c_cheb, tab, sizeof(double) * n);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_cheb_2a, two_a, sizeof(two_a));
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_cheb_at, at, sizeof(at));
-  return e;
-}
+constexpr ChebTables CHEB = cheb_tables();
+static __constant__ ChebTables c_cheb = CHEB;  // a copy per translation unit
 
 struct Ctl {
   double alpha[MAX_M + 2];
@@ -219,7 +175,7 @@ static __device__ __noinline__ void small_expm_warp(const Ctl& c, int m, int p, 
   const int ex = (int)((__float_as_uint(fmaxf(need, 1.f)) >> 23) & 0xffu) - 127;
   const float mant = __uint_as_float((__float_as_uint(fmaxf(need, 1.f)) & 0x7fffffu) | 0x3f800000u);
   const int ia = min(2 * ex + (mant > 1.41421354f ? 2 : mant > 1.f ? 1 : 0), CHEB_TABLES - 1);
-  const double g = c_cheb_2a[ia];                       // 2 / a
+  const double g = c_cheb.two_a[ia];                       // 2 / a
   double ts = g, shift = 2.0;                           // 2 X = ts K + shift
   if (s > 1) ts = g / (double)s;
   if (n2 > 0) shift = fma(-ts, (double)n2 * 0.6931471805599453, 2.0);
@@ -242,8 +198,8 @@ static __device__ __noinline__ void small_expm_warp(const Ctl& c, int m, int p, 
     if (j == 0) x[h] = 1.0;
     // the augmented rows' upper neighbours do not enter (C = 0)
   }
-  const double* const t = c_cheb + c_cheb_at[ia];
-  const int n = c_cheb_at[ia + 1] - c_cheb_at[ia];
+  const double* const t = c_cheb.c + c_cheb.at[ia];
+  const int n = c_cheb.at[ia + 1] - c_cheb.at[ia];
   if (s == 1) {
     if (lane == 0) B[0] = 1.0;
     if (two) cheb_steps<true, false>(t, n, A, B, C, x, y);
@@ -2048,7 +2004,6 @@ PhipmKernels phipm_kernels() {
   k.fn[2][1] = (void*)phipm_kernel<T, 4, true, NT>;
   k.nt = NT;
   k.adj_smem = adj_smem(NT);
-  k.load_consts = load_cheb;
   return k;
 }
 
