@@ -1,8 +1,8 @@
 // Chebyshev coefficients of the small exponential (krylov_impl.cuh), computed by the
 // compiler: a __constant__ table with a constant initialiser is part of the module,
 // on every device and before the first launch on any stream.  (Filled by a copy on
-// the host's first use it would be there for one device only, ordered with the
-// legacy stream only, and not under stream capture.)
+// the host's first use it would be there for one device only, and ordered with
+// the legacy stream, not with a non-blocking one.)
 #pragma once
 
 namespace etd {

@@ -4,8 +4,9 @@ CPU: the compiler's table against 40-digit values.  Each step of the recurrence
 rounds three times and adds positive terms, so a value is off by 3 roundings for
 every step above it at most, the normalising sum by as much and its own 512: 2050
 roundings of 2^-53.
-GPU: the first Krylov launch of a process may be one under stream capture (a table
-filled by a copy on first use could not be).
+No table is filled by a copy on first use, which would serve one device and one
+stream's order only.  GPU: the first Krylov launch of a process, under stream
+capture, gives what a plain one gives.
 """
 import ctypes
 import os
