@@ -574,15 +574,17 @@ etd_status etd_init_domain(etd_ctx* c, int species, const double* phi, const dou
   ma.diag = b.diag;
   ma.diagf = b.diagf;
   ma.facew = species == 0 ? c->facew : nullptr;
-  if (species == 0 && beta_field) (c->fp32 ? (void*&)ma.bfacef : (void*&)ma.bface) = c->bface;
+  if (species == 0 && beta_field) {
+    if (c->fp32) ma.bfacef = static_cast<float*>(c->bface);
+    else ma.bface = static_cast<double*>(c->bface);
+  }
   ma.bco = b.bco;
   ma.bpts = b.bpts;
   ma.gersh = &c->st->gersh[species];
   ma.negb = &c->st->negb[species];
   ma.st = c->st;
-  cudaError_t e = cudaSuccess;
   ma.qmeta = b.qmeta;
-  e = launch_init_domain(ca, ma, c->tile_count, b.ncomp, c->stream);
+  cudaError_t e = launch_init_domain(ca, ma, c->tile_count, b.ncomp, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "init_domain launch");
   if (c->ncomp_host) {
     e = cudaMemcpyAsync(c->ncomp_host + species, b.ncomp, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
