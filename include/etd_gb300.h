@@ -15,7 +15,8 @@
  *   - Field arguments (phi, u, beta, x, y, v0..v2) are DEVICE pointers to
  *     full-grid FP64 arrays owned by the caller; the library never frees or
  *     keeps them beyond the call, except beta_field, which must stay valid
- *     until the next etd_init_domain of that species.
+ *     and keep its values until the next etd_init_domain of that species
+ *     (etd_init_domain).
  *   - The workspace is a caller-owned device buffer of etd_workspace_bytes()
  *     bytes, 256-byte aligned; the library allocates no device memory.
  *   - Calls are asynchronous on the stream given to etd_create unless they
@@ -91,7 +92,9 @@ enum {
  *   mu[s]       Stefan coefficient of species s (boundary speed mu |grad u|)
  *   beta[s]     constant diffusion coefficient of species s, used when no
  *               beta field is given to etd_init_domain
- *   adjoint     1 to reserve the workspace of etd_adjoint_step (species 0)
+ *   adjoint     1 to reserve the workspace of etd_adjoint_step (species 0),
+ *               and ndim more full-grid fields in the Krylov vectors' precision
+ *               for the face means of a beta field
  *   scheme      time integrator of etd_step (Sec. 3.1-3.2): ETD_SCHEME_ETD1,
  *               ETD_SCHEME_ETD2 (also selected by 0), ETD_SCHEME_ETD2RK,
  *               ETD_SCHEME_ETD3RK, ETD_SCHEME_ETD4RK (these two need
@@ -150,7 +153,11 @@ void etd_destroy(etd_ctx* ctx);
  * diagonal D_p = sum_faces beta_f - sum_ghost faces beta_f w_f, with w_f the
  * ghost weight of case 2 (Eq. DirichletLineByLine) or case 3 (Eq. rbf_ubp),
  * clamped to [0, 1].  beta_field: NULL for the constant params->beta[species],
- * else a full-grid node field (face value = mean of the two nodes). */
+ * else a full-grid node field (face value = mean of the two nodes).  The
+ * diagonal, the bounds of the operator's spectrum, the sign of the field and (adjoint
+ * contexts) the face means are taken here, the field itself is read again by
+ * later calls: after a change of its values call etd_init_domain again before
+ * any other call on the species, whose results are unspecified otherwise. */
 etd_status etd_init_domain(etd_ctx* ctx, int species, const double* phi, const double* beta_field);
 
 /* One time step of every species on the current domains, by the scheme of

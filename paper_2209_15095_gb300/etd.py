@@ -206,6 +206,10 @@ class Context:
             raise EtdError(rc, self.lib.etd_last_error(self.ctx).decode())
 
     def init_domain(self, species, phi, beta_field=None):
+        """Domain set-up from phi.  beta_field's values must not change until the next
+        init_domain of the species: parts of the operator are taken from it here
+        and others read from it by later calls (after an in-place update, call
+        init_domain again first)."""
         self._beta_fields[species] = beta_field  # the library reads it until the next init
         self._check(self.lib.etd_init_domain(self.ctx, species, _ptr(phi, self.n, "phi"),
                                              _ptr(beta_field, self.n, "beta_field")))
