@@ -39,6 +39,24 @@ __device__ __forceinline__ void reaction_terms(int kind, const double* rp, doubl
   }
 }
 
+// part[blockIdx.x] = sum of v over the block, in a fixed order: warp 0 sums the staged
+// values (lane-strided, then a warp tree), so that the FP64 additions run on one
+// warp instead of every warp's shuffle tree.
+__device__ __forceinline__ void block_partial(double v, double* part) {
+  __shared__ double st[ADJ_NT];
+  st[threadIdx.x] = v;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double x0 = 0.0, x1 = 0.0;
+    for (int t = threadIdx.x; t < ADJ_NT; t += 64) {
+      x0 += st[t];
+      if (t + 32 < ADJ_NT) x1 += st[t + 32];
+    }
+    const double x = warp_sum(x0 + x1);
+    if (threadIdx.x == 0) part[blockIdx.x] = x;
+  }
+}
+
 __global__ void __launch_bounds__(ADJ_NT) adjoint_combine_kernel(const AdjointArgs a) {
   double part = 0.0;
   const long long G = a.g.size;
@@ -62,8 +80,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_combine_kernel(const AdjointAr
     a.lam[p] = lam;
     a.acc[p] = acc;
   }
-  double v[1] = {part};
-  block_partials<1>(v, a.part);
+  block_partial(part, a.part);
 }
 
 // Sums the per-block partials in a fixed order (lane-strided, then a warp tree:

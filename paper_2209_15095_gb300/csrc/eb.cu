@@ -365,15 +365,14 @@ __device__ void metadata_phase(const MetaArgs& a, int ncomp) {
 }
 
 // The whole set-up as one persistent cooperative kernel (one CTA per SM):
-//   phase 1  classify this CTA's chunk of nodes (whole 32-node words), zero
+//   phase 1  the sign plane of this CTA's chunk of nodes (whole 32-node words);
+//            after a grid barrier, classify them 32 at a time from it, zero
 //            stale vector entries where a computational node stopped being
-//            one, count computational nodes (when rows are whole words: a
-//            sign plane first, then, after a grid barrier, 32 nodes at a
-//            time from it);
+//            one, count computational nodes;
 //   phase 2  (after a grid barrier) this CTA's offset from the counts of the
 //            CTAs before it, then the grid indices of its computational nodes
 //            in grid order;
-//   phase 3  (after a second barrier) the row metadata.
+//   phase 3  (after a third barrier) the row metadata.
 template <int N>
 __device__ __forceinline__ void init_domain_body(const ClassifyArgs& ca, const MetaArgs& ma) {
   const GridDev& g = ca.g;
@@ -535,8 +534,6 @@ __global__ void __launch_bounds__(INIT_NT, 1) init_domain_kernel(const __grid_co
   barrier_done(ca.st);
 }
 
-// ints of scratch the set-up kernel needs: one count per CTA, then two bit
-// planes (computational nodes, signs of phi) of one bit per node
 template <int N>
 static void* init_fn() {
   return (void*)init_domain_kernel<N>;

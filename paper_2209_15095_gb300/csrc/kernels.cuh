@@ -43,7 +43,8 @@ struct MetaArgs {
   DevStatus* st;
 };
 
-// ints of per-CTA counts and word scratch of the set-up kernel
+// ints of scratch of the set-up kernel: one count per CTA, then two bit planes
+// (computational nodes, signs of phi) of one bit per node
 constexpr int init_scratch_ints(long long size) { return MAX_BLOCKS + 2 * (int)((size + 31) / 32); }
 cudaError_t launch_init_domain(const ClassifyArgs& ca, const MetaArgs& ma, int* tile_count, int* ncomp_dev,
                                cudaStream_t stream);

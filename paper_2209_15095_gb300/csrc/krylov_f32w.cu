@@ -5,7 +5,6 @@
 // 11.4 ms; at star3d (15.9k points) 768 threads cost the Krylov launch 15%
 // and at twoball3d (114k points per species) 11% (register spills in the
 // per-point paths), so those keep 512.
-#define ETD_RED_MAX_NT 768
 #define ETD_FACE_MEANS 0
 #include "krylov_impl.cuh"
 

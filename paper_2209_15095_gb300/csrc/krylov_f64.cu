@@ -1,7 +1,6 @@
 // Instantiation of the Krylov kernel with FP64 vectors (512 threads per CTA,
 // 128 registers per thread); also the operator-only kernel and the rounding
 // self-check.
-#define ETD_RED_MAX_NT 512
 #include "krylov_impl.cuh"
 
 namespace etd {

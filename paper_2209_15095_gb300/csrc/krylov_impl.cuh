@@ -33,8 +33,7 @@
 // This header holds the kernel; krylov_f64.cu, krylov_f32.cu and
 // krylov_f32w.cu instantiate it (FP64 with 512 threads per CTA; FP32 with
 // 512, and with 768 for problems on the 4-node groups) and krylov.cu
-// launches it.  A unit may define ETD_RED_MAX_NT (the block-reduction width)
-// before including it.
+// launches it.  A unit may define ETD_FACE_MEANS before including it.
 #pragma once
 #include "cheb.cuh"
 #include "common.cuh"
@@ -1144,9 +1143,6 @@ static __device__ __forceinline__ void quad_setup_etd2(const PhipmArgs<float>& a
   sums[2] = s2.value();
 }
 
-// The basis on the groups of 4 nodes from V_0, Z_0 and the state of a basis
-// of one vector: passes, sums and checks until the basis is accepted or
-// full.  Returns false if the kernel must stop.
 // The FP32 coefficients of pass j of the one-pass recurrence from the scale of
 // V_{j-1}, alpha_{j-1} and beta_j (one thread; every warp's own FP64 divisions
 // cost the SM 2 us per pass).
@@ -1156,6 +1152,9 @@ __device__ __forceinline__ void quad_coefs(Ctl& c, double sp, double al, double 
   c.fv2 = (float)(-bj * sp);
 }
 
+// The basis on the groups of 4 nodes from V_0, Z_0 and the state of a basis
+// of one vector: passes, sums and checks until the basis is accepted or
+// full.  Returns false if the kernel must stop.
 template <int N>
 __device__ __forceinline__ bool lanczos_quads(const PhipmArgs<float>& a, const SpeciesDev<float>& S, Ctl& c,
                                            unsigned& bar, GridSums& gs, int P) {

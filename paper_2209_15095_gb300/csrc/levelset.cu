@@ -107,19 +107,6 @@ LevelsetBufs levelset_carve(const GridDev& g, const std::function<char*(size_t)>
   return b;
 }
 
-// axis indices of node p (grids hold fewer than 2^31 nodes: 32-bit division)
-template <int N>
-__device__ __forceinline__ void coords(const GridDev& g, long long p, int* ix) {
-  unsigned rem = (unsigned)p;
-#pragma unroll
-  for (int d = 0; d < N; ++d) {
-    const unsigned st = (unsigned)g.stride[d];
-    const unsigned q = g.sdiv[d].div(rem);
-    ix[d] = (int)q;
-    rem -= q * st;
-  }
-}
-
 template <int N>
 __device__ __forceinline__ void unpack(ushort4 c, int* ix) {
   ix[0] = c.x;
@@ -386,7 +373,6 @@ __device__ __forceinline__ double grad_f32(const LsArgs& a, const StageLane<N>& 
 // ------------------------------------------------------------ work lists
 struct LsCtx {
   unsigned bar;
-  int red;
   long long wlo, whi;  // this CTA's words of the bit planes
 };
 
@@ -884,8 +870,8 @@ __device__ bool ext_sweeps(const LsArgs& a, LsCtx& c, int n, long long cap, int 
     }
     si = 2 * sw + cur;
   }
-  // the swept region of u (level 3) from FP32; the rest of the work list as
-  // the FP64 sweeps leave it (its initial values)
+  // the swept region of u (level 3) from the last sweep; the rest of the work
+  // list keeps its initial values, in FP64
   for (long long i = gtid; i < n; i += gth) {
     const long long p = __ldcg(a.b.list + i);
     a.u[p] = sweep_level(__ldcg(a.b.lflag + i)) == 3 ? (double)__ldcg(F[si] + p) : __ldcg(Q0[2] + p);
@@ -1125,7 +1111,6 @@ __global__ void __launch_bounds__(LS_NT, 1) levelset_kernel(const __grid_constan
   const GridDev& g = a.g;
   LsCtx c;
   c.bar = 0;
-  c.red = 0;
   {
     const long long nw = bit_geo(g).nw;
     const long long chunk = (nw + gridDim.x - 1) / gridDim.x;

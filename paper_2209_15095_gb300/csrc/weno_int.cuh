@@ -134,12 +134,6 @@ ETD_HD u64 recip_u(u64 w) {
   return ((u64)r0 << 32) + (u64)c;
 }
 
-// (x y) >> 62 for |x| < 2^60 (signed) and a signed |y| < 2^63, to within 2 units
-ETD_HD i64 mul62(i64 x, i64 y) {
-  const U128 p = mul128(x, y);
-  return (i64)(p.hi << 2 | p.lo >> 62);
-}
-
 // 12 Phi(a, b, c, d) of Jiang & Peng's form (levelset.cu, weno5_terms) from
 // second differences in units 2^-S:
 //   12 Phi = (4 A X + V Y) / W,  A = d1 d2, B = d0 d2, C = d0 d1,
