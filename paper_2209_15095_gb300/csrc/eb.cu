@@ -231,6 +231,7 @@ __device__ void metadata_phase(const MetaArgs& a, int ncomp) {
   // FP64 face sums (FP64 warp instructions are what this phase spends)
   const bool cbeta = a.beta_field == nullptr;
   const double D_int = (double)FPR * a.beta_c;
+  const float Df_int = (float)D_int;
   const unsigned row_mask = ((1u << FPR) - 1u) << lead;
   bool seen_interior = false;
   for (long long w = (long long)blockIdx.x + (long long)gridDim.x * (threadIdx.x >> 5); w * RPW < ncomp;
@@ -332,7 +333,8 @@ __device__ void metadata_phase(const MetaArgs& a, int ncomp) {
     const bool interior = cbeta && (fc & row_mask) == row_mask;
     // the face sums only where some row of this warp iteration has a ghost face
     const unsigned need = __ballot_sync(0xffffffffu, act && f == 0 && !interior);
-    double D = D_int, off = D_int;
+    double D = D_int;
+    float Df = Df_int;
     if (need) {
       double Ds = 0.0, os = 0.0;
 #pragma unroll
@@ -340,15 +342,18 @@ __device__ void metadata_phase(const MetaArgs& a, int ncomp) {
         Ds += __shfl_sync(0xffffffffu, cD, lead + j);
         os += __shfl_sync(0xffffffffu, cOff, lead + j);
       }
+      // (all FP64 work of a row in this block: beside the stores below the compiler
+      // predicates the sum, the maximum and the conversion, and predicated off they still
+      // take their issue slots in every interior iteration: 46M points 3.09 ms, now 2.68)
       if (!interior) {
         D = Ds;
-        off = os;
+        Df = (float)Ds;
+        if (act && f == 0) gmax = fmax(gmax, Ds + os);
       }
     }
     if (act && f == 0) {
       a.diag[k] = D;
-      if (a.diagf) a.diagf[k] = (float)D;
-      if (!interior) gmax = fmax(gmax, D + off);
+      if (a.diagf) a.diagf[k] = Df;
       seen_interior = seen_interior || interior;
     }
   }
