@@ -641,26 +641,40 @@ __device__ __forceinline__ T tabs(T x) {
 // than SW_CACHE times the grid's threads) load them in every pass.  Measured
 // on regions of one to two entries per thread (4D, FP32, 83k nodes): 4.8 us a
 // pass with every entry loaded in every pass, 3.1 with the entries kept (3D,
-// 256^3: 3.55 and 2.34).
+// 256^3: 3.55 and 2.34).  Of many entries per thread the loads bound a pass: an
+// advancing launch of the mixed variant at 80^4 (2M nodes) 13.2 ms (17.0 with the
+// arguments' pointers read again after every store, 13.8 inlined into the kernel
+// without kept entries), at 512^3 10.1 (11.3, 10.3).
 template <int N, typename T>
 __device__ __noinline__ bool sweep_single(const LsArgs& a, LsCtx& c, long long len, long long cap, int K, T dtau, T dth,
                                           T* const* X, const T* __restrict__ src) {
   constexpr int SW_CACHE = 2;
-  const GridDev& g = a.g;
+  // pointers and extents in registers: through the launch's arguments they would be
+  // read again after every store
+  const int* __restrict__ const slist = a.b.slist;
+  const int* __restrict__ const list = a.b.list;
+  const ushort4* __restrict__ const lcoord = a.b.lcoord;
+  const double* __restrict__ const nrm = a.b.nrm;
+  int gn[N], gst[N];
+#pragma unroll
+  for (int d = 0; d < N; ++d) {
+    gn[d] = a.g.n[d] - 1;
+    gst[d] = (int)a.g.stride[d];
+  }
   const long long gth = (long long)gridDim.x * blockDim.x, jt = dealt_tid();
   int cp[SW_CACHE], cup[SW_CACHE][N];
   T cq[SW_CACHE], cds[SW_CACHE], cc0[SW_CACHE], ca[SW_CACHE][N];
   const auto load = [&](long long j, int& p, int* up, T& ds, T& c0, T* ad) {
-    const long long i = __ldcg(a.b.slist + j);
-    p = __ldcg(a.b.list + i);
+    const int i = __ldcg(slist + j);
+    p = __ldcg(list + i);
     ds = src ? dtau * __ldcg(src + p) : T(0);
     int ix[N];
-    unpack<N>(__ldcg(a.b.lcoord + i), ix);
+    unpack<N>(__ldcg(lcoord + i), ix);
     T asum = T(0);
 #pragma unroll
     for (int d = 0; d < N; ++d) {
-      const double nd = __ldcg(a.b.nrm + d * cap + i);
-      up[d] = (int)nbr(g, p, ix, d, nd > 0.0 ? -1 : 1);
+      const double nd = __ldcg(nrm + d * cap + i);
+      up[d] = nd > 0.0 ? (ix[d] > 0 ? p - gst[d] : p) : (ix[d] < gn[d] ? p + gst[d] : p);
       ad[d] = dth * tabs((T)nd);
       asum += ad[d];
     }
