@@ -960,12 +960,14 @@ __device__ __forceinline__ void stage_push(const LsArgs& a, int i, bool front) {
 
 // How the stage list is dealt: chunks of warps' work, round-robin over the
 // CTAs (every SM gets its share of each kind).  Front entries go a lane each,
-// or, where they then still make one round of the warps at most, an axis per
-// lane (32 / N entries per warp): the same instructions in all, a third (3D) of
-// the dependent chain per warp.  Back entries go a lane each in what rounds
-// follow, and do not count: a reinitialisation of the mixed variant, with few
-// front entries among many, took 1.71 instead of 1.35 ms on a steep phi at 200^3 where
-// they did (five steps of the 4D ellipsoid at 48^4 3.66 instead of 3.42 ms).
+// or, where they then make one round of the warps at most and the whole list no
+// more rounds than otherwise, an axis per lane (32 / N entries per warp): the
+// same instructions in all, a third (3D) of the dependent chain per warp.  Back
+// entries go a lane each in what rounds follow.  Mixed reinitialisations, with few
+// front entries among many: asking for one round of all entries cost 1.71 instead
+// of 1.35 ms on a steep phi at 200^3 and 3.66 instead of 3.42 ms in five steps of
+// the 4D ellipsoid at 48^4; asking for the front entries' round alone added a round
+// of the others at some sizes (139^3 0.70 instead of 0.66 ms).
 template <int N>
 struct StageDeal {
   static constexpr int NPW = 32 / N;  // split entries per warp
@@ -976,9 +978,9 @@ struct StageDeal {
     nb = __ldcg(a.b.count + 2);
     warp0 = (int)blockIdx.x + (int)gridDim.x * (int)(threadIdx.x >> 5);
     wstride = (int)gridDim.x * (int)(blockDim.x >> 5);
-    const int cb = (nb + 31) / 32, cs = (nf + NPW - 1) / NPW;
-    split = cs <= wstride;
-    cf = split ? cs : (nf + 31) / 32;
+    const int cb = (nb + 31) / 32, cs = (nf + NPW - 1) / NPW, cw = (nf + 31) / 32;
+    split = cs <= wstride && (cs + cb - 1) / wstride <= (cw + cb - 1) / wstride;
+    cf = split ? cs : cw;
     nchunk = cf + cb;
   }
   // this lane's entry of a chunk
