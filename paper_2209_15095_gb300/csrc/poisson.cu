@@ -31,8 +31,8 @@ constexpr int PS_NT = 512;
 // thread 15.9 / 16.0, 4.5 20.7 / 19.2, 17.5 62.2 / 51.4, 2D 2.4 13.1 / 14.5, 4.9 18.8 /
 // 18.4; node field (the means cost more than either): 3D 2.8 18.5 / 20.3, 4.5 26.5 /
 // 26.5, 17.5 93.2 / 85.8, 2D 4.9 22.9 / 23.8, 8.1 34.8 / 35.0.
-template <bool NODE>
-constexpr int PS_FUSED_PER = NODE ? 5 : 3;
+template <int N, bool NODE>
+constexpr int PS_FUSED_PER = N == 2 ? (NODE ? 8 : 4) : NODE ? 5 : 3;
 
 // A computational point of the stencil: grid index (-1: none), diagonal and,
 // with a node field (NODE), face coefficients.  NODE is a template argument: a
@@ -95,7 +95,7 @@ __device__ __forceinline__ void poisson_body(const PoissonArgs& a) {
   GridSums gs(a.part);
   double* const x = S.Yc;             // compact: iterate
   double* const q = (double*)S.V2c;   // compact: A p
-  const bool fused = ncomp <= PS_FUSED_PER<NODE> * gth;
+  const bool fused = ncomp <= PS_FUSED_PER<N, NODE> * gth;
   double* const r = (double*)(fused ? S.Z[0] : S.V1c);  // residual: grid (zero off the set), or compact
   double* const P[2] = {(double*)S.Yg, (double*)S.W1g};  // grid: search direction (zero off the set)
   __shared__ double s_alpha, s_beta, s_rr, s_stop, s_stop2;
