@@ -979,7 +979,9 @@ struct StageDeal {
     warp0 = (int)blockIdx.x + (int)gridDim.x * (int)(threadIdx.x >> 5);
     wstride = (int)gridDim.x * (int)(blockDim.x >> 5);
     const int cb = (nb + 31) / 32, cs = (nf + NPW - 1) / NPW, cw = (nf + 31) / 32;
-    split = cs <= wstride && (cs + cb - 1) / wstride <= (cw + cb - 1) / wstride;
+    int cap = wstride;  // whole rounds (counted: two divisions here cost the stages 1.5%)
+    while (cap < cw + cb) cap += wstride;
+    split = cs <= wstride && cs + cb <= cap;
     cf = split ? cs : cw;
     nchunk = cf + cb;
   }
